@@ -62,10 +62,11 @@ long long conv_plan(int taps3d, int H, int cpin, int cin, int cout, int flip, Co
 // Packs njobs layers (jobs: device array) from params into out in one launch.
 int conv_pack_jobs(const ConvPackJob *jobs, int njobs, long long max_nelem, const float *params, uint8_t *out,
                    cudaStream_t st);
-// Looks up (once per device) the device address of back_project_noalloc's fixed
-// scratch array on `dev`, the current device. geometry_create calls it so that the
-// module holding the array is loaded, and the array placed, when the geometry is made.
-int noalloc_prime(int dev);
+// Called by geometry_create on `dev`, the current device: sets the projector kernels'
+// shared-memory limits (so that no call has to) and looks up the device address of
+// back_project_noalloc's fixed scratch array, so that the module holding the array is
+// loaded, and the array placed, when the geometry is made.
+int projector_prime(int dev);
 // Staged (TMA) forward: returns 1 if it ran, 0 if the direct kernel must be used.
 int forward_staged(const cbct_geom *g, const float *vol, float *proj, int batch, int accumulate, cudaStream_t st);
 int choose_forward_cfg(double need_b, double need_z);

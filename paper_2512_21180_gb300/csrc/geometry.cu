@@ -253,6 +253,13 @@ extern "C" int geometry_create(const cbct_geom_desc *desc, cbct_geom **out) {
         geometry_destroy(g);
         return cuda_fail(e, "geometry_create: table upload");
     }
+    // the projector kernels' shared-memory limits and the fixed scratch array of
+    // back_project_noalloc on this device: the lookup loads the projector module (and so places
+    // the array) here, so that the no-allocation entry point itself never reaches the allocator
+    {
+        int rc = cbct::projector_prime(dev);
+        if (rc != 0) { geometry_destroy(g); return rc; }
+    }
     GeomDev &v = g->dev;
     v.n[0] = d.nx; v.n[1] = d.ny; v.n[2] = d.nz;
     v.nu = d.nu; v.nv = d.nv; v.na = d.n_angles;
@@ -274,13 +281,6 @@ extern "C" int geometry_create(const cbct_geom_desc *desc, cbct_geom **out) {
         if (!(nrm > 0.0)) { geometry_destroy(g); return fail(CBCT_EINVAL, "geometry_create: ||P|| is zero"); }
         v.scaled = 1.0 / nrm;
         v.scale = (float)v.scaled;
-    }
-    // resolve the fixed scratch array of back_project_noalloc on this device now: the
-    // lookup loads the projector module (and so places the array) here, so that the
-    // no-allocation entry point itself never reaches the allocator
-    {
-        int rc = cbct::noalloc_prime(dev);
-        if (rc != 0) { geometry_destroy(g); return rc; }
     }
     *out = g;
     return 0;

@@ -14,7 +14,7 @@
 // projection beforehand (k_weight_rays) so the gather needs no square root.
 // This kernel serves the FP64 instantiation and geometries whose principal-axis
 // columns do not form intervals; FP32 calls otherwise use the segment gather
-// k_backproject_v3 further down, which visits the same triples.
+// k_backproject_seg further down, which visits the same triples.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -22,6 +22,7 @@
 
 #include "common.cuh"
 #include "geom_impl.h"
+#include "tma.cuh"
 
 namespace cbct {
 
@@ -96,7 +97,8 @@ __global__ void __launch_bounds__(256) k_forward(GeomDev g, const T *__restrict_
 
 // pw = proj * step(ray) * scale (* colw[column] when colw is given)
 template <typename T>
-__global__ void k_weight_rays(GeomDev g, const T *__restrict__ proj, T *__restrict__ pw, const T *__restrict__ colw) {
+__global__ void k_weight_rays(GeomDev g, const T *__restrict__ proj, T *__restrict__ pw, const T *__restrict__ colw,
+                              int pitch) {
     const int iu = blockIdx.x * 32 + threadIdx.x;
     const int iv = blockIdx.y * 8 + threadIdx.y;
     const int k = blockIdx.z % g.na, b = blockIdx.z / g.na;
@@ -107,9 +109,9 @@ __global__ void k_weight_rays(GeomDev g, const T *__restrict__ proj, T *__restri
     ray_row(g, c, rz_of<T>(g, iv), dqz, qcz);
     T scale;
     if constexpr (sizeof(T) == 4) scale = g.scale; else scale = g.scaled;
-    const long long o = (((long long)b * g.na + k) * g.nv + iv) * g.nu + iu;
-    const T v = proj[o] * ray_step<T>(g, a, c.dqb, dqz) * scale;
-    pw[o] = colw ? v * colw[iu] : v;
+    const long long row = ((long long)b * g.na + k) * g.nv + iv;
+    const T v = proj[row * g.nu + iu] * ray_step<T>(g, a, c.dqb, dqz) * scale;
+    pw[row * pitch + iu] = colw ? v * colw[iu] : v;
 }
 
 // Detector column (continuous) hit by the ray from the source through the xy
@@ -209,206 +211,326 @@ __global__ void __launch_bounds__(256) k_backproject(GeomDev g, const T *__restr
 }
 
 // Segment gather (FP32, geometries whose x- and y-principal columns form intervals).
-// CTA = brick of 16 x 16 voxel columns x 8 voxels in z, 288 threads. For the rays
-// of principal axis a at angle k, plane i of the brick is crossed at
-// q_b(u) = fma(di, dqb(u), qcb(u)), monotone in the detector column u. The columns
-// with floor(q_b) = s form segment s of the plane; their samples lie between voxels
-// s and s + 1 with weights 1 - frac(q_b) and frac(q_b). Thread (segment, plane)
-// sweeps the rows of each of its columns once, summing the rows of every unit
-// z-interval (L, L + 1] as S0 = sum p and S1 = sum p (q_z - L) (lower voxel
-// S0 - S1, upper voxel S1), and accumulates SA[z] for voxel s and SB[z] for voxel
-// s + 1. A thread's two voxel runs depend on the axis only, so the angles run inside
-// one sweep per principal axis and SA, SB stay in registers over all of them; after
-// each sweep every voxel adds the SA of its own segment, then (after a barrier) the SB
-// of the segment below, to its shared accumulator — a fixed order, so the result does
-// not depend on scheduling, and no barrier or shared-memory traffic per angle.
-// The kernel is bound by load latency, which shapes the loops: a thread first
-// narrows its candidate columns to the first and last column of its segment (so
-// the lanes of a warp run their useful columns in the same iterations); a row's
-// z-coordinate is the affine q_z(v) = voff + v step of the row index (rz(v) =
-// rz_0 + v EV_z), so no table load sits between two intervals; and the rows of
-// an interval go through a fixed block of five predicated loads (3 to 5 rows per
-// interval at these magnifications) plus a loop for longer intervals, which makes
-// the (kZ3 + 1)-interval sweep straight-line code whose loads overlap.
-// The panel width is a template parameter for common widths (256, 512, 1024 columns): the five
-// row loads of an interval then sit at constant offsets from one row pointer, which took the
-// clinical adjoint from 23.3 to 19.6 ms (CUDA events, bit-identical output).
-// Bricks 8 voxels tall with four CTAs per SM (registers capped at 56, no spills): with the
-// width-specialised loads the kernel is bound by load latency more than by issue, and the
-// fourth CTA's warps hide it. Clinical adjoint (CUDA events): 18.3 ms, against 19.6 with
-// 12-voxel bricks at three CTAs, 19.7 with 8-voxel bricks at three, 19.0 with 10 at four,
-// 20.0 with 6 at four, 28.4 with 12 at four and 23.3 with 8 at five (spills). Before the
-// width-specialised loads 12-voxel bricks at three CTAs had been best (23.7 ms; 24.5 with 8,
-// 26.0 with 6, 31.5 with 4, 26.8 with 16; capped registers slower).
-constexpr int kB3 = 16, kZ3 = 8, kThreads3 = 288;
-constexpr int kVacc3 = kZ3 * kB3 * (kB3 + 1);  // [z][y][x], y stride 17 (bank-conflict free both ways)
-constexpr size_t kSmem3 = sizeof(float) * kVacc3;
+// CTA = brick of 16 x 16 voxel columns x 8 voxels in z, 288 threads. For the rays of
+// principal axis a at angle k, plane i of the brick is crossed at q_b(u) =
+// fma(di, dqb(u), qcb(u)), monotone in the detector column u. The columns with
+// floor(q_b) = s form segment s of the plane; their samples lie between voxels s and
+// s + 1 with weights 1 - frac(q_b) and frac(q_b). Thread (segment, plane) accumulates
+// SA[z] for voxel s and SB[z] for voxel s + 1 in registers over all angles of one
+// principal axis; after each sweep every voxel takes the SA of its own segment, then
+// (after a barrier) the SB of the segment below — a fixed order, so the result does not
+// depend on scheduling.
+//
+// Along a column the samples of plane i have q_z affine in the row, and a row in the unit
+// interval (L, L + 1] weighs L + 1 - q_z on voxel L and q_z - L on voxel L + 1: each interval
+// needs only sum p and sum p row over its rows. Neighbouring planes and segments of a
+// brick ask for overlapping rows of the same columns (about 60 requests per loaded value),
+// so the tile of the projection that the brick sees at one angle is loaded once (TMA, the
+// next tile in flight while this one is summed), turned into prefix sums (sum p,
+// sum (row - h) p) down each column, and every interval is the difference of two entries:
+// 12 instructions instead of a run of predicated row loads (3 to 5 rows per interval at
+// these magnifications). The sums start at the tile's middle row h and run outwards, so
+// they span at most half a tile (26 rows) of one column: FP32 rounding stays that of a
+// short sum, and the measured error against 64 bits is the row-by-row kernel's (clinical
+// 3.5e-7 both). Bounded by instruction issue: about 3/4 of the instructions are the
+// intervals, 1/8 the prefix sums. Back projection by CUDA events, before -> after:
+// clinical 17.4 -> 9.3 ms, 2 x 128^3 / 200 angles 3.79 -> 1.68 ms, 181 x 167 x 93 / 150 angles
+// 4.12 -> 1.26 ms, 64^3 / 64 angles 126 -> 69 us.
+//
+// A tile whose sums are not finite (an infinite or NaN pixel, or an overflow) is summed row
+// by row instead, so such a pixel reaches the voxels its ray touches and no others. A brick
+// whose footprint exceeds the tile takes several tiles per angle: the intervals are linear in
+// the rows, so a tile that holds part of an interval adds its part.
+//
+// Tile 112 x 52: the largest that lets three CTAs share an SM (clinical 9.3 ms; 96 x 60 9.7,
+// 120 x 48 9.8, 128 x 46 10.0, 80 x 64 11.0 with more tiles split in columns; 112 x 56 at two
+// CTAs per SM 10.9; without the TMA stage, reading the rows from L2, 10.6 at three and 12.5
+// at four CTAs of 56 registers).
+constexpr int kB3 = 16, kZ3 = 8, kThreads3 = 288, kWarps3 = kThreads3 / 32;
+constexpr int kBC = 112, kBR = 52;       // tile: detector columns x rows
+constexpr int kEP = kBC + 1;            // pitch of the prefix sums (entries), odd: rows fall into different banks
+constexpr int kChunk3 = 128;            // angles listed at a time
+constexpr size_t kE3Bytes = (((size_t)(kBR + 1) * kEP * 8) + 127) & ~(size_t)127;
+constexpr size_t kRaw3Bytes = (size_t)kBC * kBR * 4;
+static_assert(kBC <= 32 * (kWarps3 / 2), "two warps per 32 columns");
+static_assert(kRaw3Bytes % 128 == 0 && (size_t)kZ3 * kB3 * (kB3 + 1) * 4 <= kE3Bytes, "tile layout");
+constexpr size_t kSmem3 = 128 + kRaw3Bytes + kE3Bytes;
 
-// NU > 0 fixes the panel width at compile time, so the rows of an interval are loaded at
-// constant offsets (rr NU floats) from one row pointer; NU = 0 reads it from the geometry.
-template <int NU>
-__global__ void __launch_bounds__(kThreads3, 4) k_backproject_v3(GeomDev g, const float *__restrict__ pw,
-                                                                 float *__restrict__ vol, int accumulate,
-                                                                 int nparts, float *__restrict__ partial) {
-    extern __shared__ float sm3[];
-    float *vacc = sm3;
-    const int tid = threadIdx.x;
+// Columns [u0, u1] and rows [v0, v1] of one angle that reach a brick.
+struct AngleSpan {
+    int k, u0, u1, v0, v1;
+};
+
+__device__ __forceinline__ bool all_finite(float a, float b) { return fabsf(a) < INFINITY && fabsf(b) < INFINITY; }
+
+__global__ void __launch_bounds__(kThreads3, 3)
+    k_backproject_seg(const __grid_constant__ CUtensorMap pmap, GeomDev g, const float *__restrict__ pw, int pitch,
+                      float *__restrict__ vol, int accumulate, int nparts, float *__restrict__ partial, int *status) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    unsigned char *sm = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
+    float *raw = reinterpret_cast<float *>(sm);
+    float2 *E = reinterpret_cast<float2 *>(sm + kRaw3Bytes);
+    float *vacc = reinterpret_cast<float *>(E);  // between the sweeps
+    __shared__ AngleSpan list[kChunk3];
+    __shared__ int wcount[kWarps3];
+    __shared__ uint64_t full;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int il = tid & 15, seg = tid >> 4;  // plane il of the brick; segment j0 - 1 + seg
     const bool item = seg <= kB3;             // 17 segments x 16 planes
     const int x0 = blockIdx.x * kB3, y0 = blockIdx.y * kB3;
     const int nzb = (g.n[2] + kZ3 - 1) / kZ3;
     const int part = blockIdx.z % nparts, zb = blockIdx.z / nparts;
     const int z0 = (zb % nzb) * kZ3, b = zb / nzb;
-    const int nx = g.n[0], ny = g.n[1], nz = g.n[2], nu = NU > 0 ? NU : g.nu, nv = g.nv;
+    const int nx = g.n[0], ny = g.n[1], nz = g.n[2], nv = g.nv;
     const int k_begin = (int)((long long)g.na * part / nparts);
-    int k_end = (int)((long long)g.na * (part + 1) / nparts);
-    __shared__ int s_reach;
-    if (tid == 0) s_reach = 0;
-    for (int e = tid; e < kVacc3; e += kThreads3) vacc[e] = 0.f;
-    __syncthreads();
+    const int k_end = (int)((long long)g.na * (part + 1) / nparts);
     const float Sz = g.Sz;
     const float rz0 = g.rz32[0], drz = g.f32[0].EV[2], inv_drz = 1.0f / drz;
-    const float *PB = pw + (long long)b * g.na * nv * nu;
-    {
-        // Does any panel row reach the brick's support (the brick and one voxel around it)
-        // at an angle of this part? The source-to-panel parameter t of a point is affine in
-        // its (x, y), so over the support it lies between its values at the four corners;
-        // the rows that meet z in (zlo, zhi) at t lie between zlo / t and zhi / t, and
-        // those are monotone in t. Two rows of margin, as in the per-column test below; a
-        // non-finite value counts as reachable. Bricks no row reaches skip the angle loop
-        // and write zeros.
-        const float zlo = (float)(z0 - 1) - Sz, zhi = (float)(z0 + kZ3) - Sz;
-        const float cx[2] = {(float)(x0 - 1), (float)(x0 + kB3)}, cy[2] = {(float)(y0 - 1), (float)(y0 + kB3)};
-        bool any = false;
-        for (int k = k_begin + tid; k < k_end && !any; k += kThreads3) {
-            const Frame32 &F = g.f32[k];
-            const float den = F.EU[0] * F.D0S[1] - F.EU[1] * F.D0S[0];
-            float tmin = INFINITY, tmax = -INFINITY;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const float t = __fdividef(F.EU[0] * (cy[c >> 1] - F.S[1]) - F.EU[1] * (cx[c & 1] - F.S[0]), den);
-                tmin = fminf(tmin, t);
-                tmax = fmaxf(tmax, t);
-            }
-            if (tmax <= 0.f) continue;  // behind the source
-            const float t1 = fmaxf(tmin, 1e-6f);
-            const float rlo = fminf(__fdividef(zlo, t1), __fdividef(zlo, tmax));
-            const float rhi = fmaxf(__fdividef(zhi, t1), __fdividef(zhi, tmax));
-            const float va = (rlo - rz0) * inv_drz, vb = (rhi - rz0) * inv_drz;
-            if (!(fmaxf(va, vb) + 2.f < 0.f || fminf(va, vb) - 2.f > (float)(nv - 1))) any = true;
-        }
-        if (any) s_reach = 1;
+    if (tid == 0) {
+        mbar_init(&full, 1);
+        fence_mbar_init();
+        prefetch_tmap(&pmap);
     }
-    __syncthreads();
-    if (!s_reach) k_end = k_begin;
+    uint32_t phase = 0;
+    bool ok = true;
+    constexpr int kKeep = (kZ3 * kB3 * kB3 + kThreads3 - 1) / kThreads3;
+    float keep[kKeep];
+#pragma unroll
+    for (int j = 0; j < kKeep; ++j) keep[j] = 0.f;
 
 #pragma unroll 1
     for (int a = 0; a < 2; ++a) {
-        const int j0 = a == 0 ? y0 : x0;
-        const int i = (a == 0 ? x0 : y0) + il, s = j0 - 1 + seg;
+        const int i0 = a == 0 ? x0 : y0, j0 = a == 0 ? y0 : x0;
+        const int i = i0 + il, s = j0 - 1 + seg;
         const bool mine = item && i < g.n[a] && s < g.n[1 - a];
         const float di = (float)i - 0.5f * (float)(g.n[a] - 1);
         float SA[kZ3], SB[kZ3];
 #pragma unroll
         for (int m = 0; m < kZ3; ++m) SA[m] = SB[m] = 0.f;
 #pragma unroll 1
-        for (int k = k_begin; k < k_end; ++k) {
-            const Frame32 &F = g.f32[k];
-            const int alo = a == 0 ? F.ux_lo : F.uy_lo, ahi = a == 0 ? F.ux_hi : F.uy_hi;
-            if (alo > ahi || !mine) continue;
-            const float *Pk = PB + (long long)k * nv * nu;
-            // candidate columns for q_b in [s, s + 1), one column of margin (which also covers
-            // the approximate divisions here and in the z-run test below: the exact test on
-            // floor(q_b) decides which columns contribute)
-            float u1, u2;
-            if (a == 0) { u1 = column_of_approx(F, (float)i, (float)s); u2 = column_of_approx(F, (float)i, (float)(s + 1)); }
-            else { u1 = column_of_approx(F, (float)s, (float)i); u2 = column_of_approx(F, (float)(s + 1), (float)i); }
-            int ulo = alo, uhi = ahi;
-            if (isfinite(u1) && isfinite(u2)) {
-                ulo = max(ulo, (int)floorf(fmaxf(fminf(u1, u2), -1.0e6f)) - 1);
-                uhi = min(uhi, (int)ceilf(fminf(fmaxf(u1, u2), 1.0e6f)) + 1);
-            }
-            if (ulo <= uhi) {
-                // skip the columns when no row of the panel reaches the z-run
-                const ColT<float> cl = col_of<float>(g, k, ulo), ch = col_of<float>(g, k, uhi);
-                const float tl = fma_rn(di, cl.inv, cl.tc), th = fma_rn(di, ch.inv, ch.tc);
-                const float tmin = fminf(tl, th), tmax = fmaxf(tl, th);
-                const float zlo = (float)(z0 - 1) - Sz, zhi = (float)(z0 + kZ3) - Sz;
-                const float t1 = fmaxf(tmin, 1e-6f);
-                const float rlo = fminf(__fdividef(zlo, t1), __fdividef(zlo, tmax));
-                const float rhi = fmaxf(__fdividef(zhi, t1), __fdividef(zhi, tmax));
-                const float vlo = (rlo - rz0) * inv_drz - 2.f, vhi = (rhi - rz0) * inv_drz + 2.f;
-                if (!(tmax > 0.f) || vhi < 0.f || vlo > (float)(nv - 1)) uhi = ulo - 1;
-            }
-            {  // first and last column of the segment
-                int ua = uhi + 1, ub = uhi;
-#pragma unroll 1
-                for (int u = ulo; u <= uhi; ++u) {
-                    const ColT<float> c = col_of<float>(g, k, u);
-                    const float t = fma_rn(di, c.inv, c.tc);
-                    const float qb = fma_rn(di, c.dqb, c.qcb);
-                    if (t > 0.f && t < 1.f && floorf(qb) == (float)s) { ua = min(ua, u); ub = u; }
-                }
-                ulo = ua;
-                uhi = ub;
-            }
-#pragma unroll 1
-            for (int u = ulo; u <= uhi; ++u) {
-                const ColT<float> c = col_of<float>(g, k, u);
-                const float t = fma_rn(di, c.inv, c.tc);
-                if (!(t > 0.f && t < 1.f)) continue;
-                const float qb = fma_rn(di, c.dqb, c.qcb);
-                const float fb = floorf(qb);
-                if (fb != (float)s) continue;  // the column belongs to another segment
-                const float wu = qb - fb, wl = 1.0f - wu;
-                const float step = t * drz, irs = 1.0f / step, voff = fmaf(t, rz0, Sz);
-                // sample z of row v relative to z0 - 1: v step + voffz; the first row whose
-                // sample lies above z0 - 1 + m is floor((m - voffz) / step) + 1, and clamping
-                // the quotient to [-1, nv - 1] before the floor keeps it in [0, nv]
-                const float voffz = voff - (float)(z0 - 1), vbase = -voffz * irs;
-                const float vmax = (float)(nv - 1);
-                auto row_above = [&](int m) {
-                    return __float2int_rd(fminf(fmaxf(fmaf((float)m, irs, vbase), -1.0f), vmax)) + 1;
-                };
-                const float *Pu = Pk + u;
-                int va = row_above(0);
-                float carry = 0.f;  // upper-voxel share of the previous interval
+        for (int kc = k_begin; kc < k_end; kc += kChunk3) {
+            // list the angles of this chunk that reach the brick, in order
+            __syncthreads();
+            AngleSpan sp{0, 0, -1, 0, -1};
+            if (tid < kChunk3 && kc + tid < k_end) {
+                const Frame32 &F = g.f32[kc + tid];
+                const int alo = a == 0 ? F.ux_lo : F.uy_lo, ahi = a == 0 ? F.ux_hi : F.uy_hi;
+                if (alo <= ahi) {
+                    // the support (planes i0 .. i0 + 15, in-plane j0 - 1 .. j0 + 16) seen from the source
+                    const float den = F.EU[0] * F.D0S[1] - F.EU[1] * F.D0S[0];
+                    float tmin = INFINITY, tmax = -INFINITY, umin = INFINITY, umax = -INFINITY;
+                    bool fin = true;
 #pragma unroll
-                for (int m = 0; m < kZ3 + 1; ++m) {
-                    const int ve = row_above(m + 1);
-                    float S0 = 0.f, S1 = 0.f;
-                    if (va < ve) {
-                        float qf = fmaf((float)va, step, voffz) - (float)m;
-                        const float *pp = Pu + (long long)va * nu;
-                        const int n = ve - va;
-                        float T = 0.f;  // sum of rr p: S1 = qf S0 + step T
-#pragma unroll
-                        for (int rr = 0; rr < 5; ++rr) {
-                            const float p = rr < n ? __ldg(pp + rr * nu) : 0.f;
-                            S0 += p;
-                            if (rr > 0) T = fmaf((float)rr, p, T);
-                        }
-#pragma unroll 1
-                        for (int rr = 5; rr < n; ++rr) {
-                            const float p = __ldg(pp + rr * nu);
-                            S0 += p;
-                            T = fmaf((float)rr, p, T);
-                        }
-                        S1 = fmaf(qf, S0, step * T);
+                    for (int c = 0; c < 4; ++c) {
+                        const float ci = (float)(i0 + (c & 1) * (kB3 - 1)), cj = (float)(j0 - 1 + (c >> 1) * (kB3 + 1));
+                        const float px = a == 0 ? ci : cj, py = a == 0 ? cj : ci;
+                        const float t = __fdividef(F.EU[0] * (py - F.S[1]) - F.EU[1] * (px - F.S[0]), den);
+                        const float u = column_of_approx(F, px, py);
+                        fin = fin && all_finite(t, u);
+                        tmin = fminf(tmin, t);
+                        tmax = fmaxf(tmax, t);
+                        umin = fminf(umin, u);
+                        umax = fmaxf(umax, u);
                     }
-                    // voxel z0 - 1 + m: upper share of interval m - 1, lower share of interval m
-                    if (m >= 1) {
-                        const float R = carry + S0 - S1;
-                        SA[m - 1] = fmaf(wl, R, SA[m - 1]);
-                        SB[m - 1] = fmaf(wu, R, SB[m - 1]);
+                    int ulo = alo, uhi = ahi, vlo = 0, vhi = nv - 1;
+                    // a support that reaches the source's own plane has no such bounds: whole panel
+                    if (fin && tmin > 1e-3f) {
+                        ulo = max(alo, (int)floorf(fmaxf(umin, -1.0e6f)) - 1);
+                        uhi = min(ahi, (int)ceilf(fminf(umax, 1.0e6f)) + 1);
+                        const float zlo = (float)(z0 - 1) - Sz, zhi = (float)(z0 + kZ3) - Sz;
+                        const float rlo = fminf(__fdividef(zlo, tmin), __fdividef(zlo, tmax));
+                        const float rhi = fmaxf(__fdividef(zhi, tmin), __fdividef(zhi, tmax));
+                        const float va = (rlo - rz0) * inv_drz, vb = (rhi - rz0) * inv_drz;
+                        vlo = max(0, (int)floorf(fmaxf(fminf(va, vb), -1.0e6f)) - 1);
+                        vhi = min(nv - 1, (int)ceilf(fminf(fmaxf(va, vb), 1.0e6f)) + 1);
+                    } else if (fin && tmax <= 0.f) {
+                        uhi = ulo - 1;  // behind the source
                     }
-                    carry = S1;
-                    va = ve;
+                    if (ulo <= uhi && vlo <= vhi)
+                        sp = AngleSpan{kc + tid, ulo & ~3, uhi, vlo, vhi};
                 }
             }
+            const bool has = sp.u0 <= sp.u1 && sp.v0 <= sp.v1;
+            const unsigned bal = __ballot_sync(0xffffffffu, has);
+            if (lane == 0) wcount[warp] = __popc(bal);
+            __syncthreads();
+            int at = __popc(bal & ((1u << lane) - 1u)), nlist = 0;
+            for (int w = 0; w < kWarps3; ++w) {
+                if (w < warp) at += wcount[w];
+                nlist += wcount[w];
+            }
+            if (has) list[at] = sp;
+            __syncthreads();
+            if (nlist == 0) continue;
+
+            // tiles of the listed angles: (angle n, columns tu .., rows tv ..); the box of the next
+            // tile is on its way while the current one is summed
+            int n = 0, tu = list[0].u0, tv = list[0].v0;
+            if (tid == 0) {
+                mbar_arrive_expect_tx(&full, (uint32_t)kRaw3Bytes);
+                tma_load_3d(raw, &pmap, tu, tv, b * g.na + list[0].k, &full);
+            }
+            while (n < nlist) {
+                const AngleSpan cur = list[n];
+                const int k = cur.k, nc = min(kBC, cur.u1 - tu + 1), nr = min(kBR, cur.v1 - tv + 1);
+                const int u0 = tu, v0 = tv;
+                // next tile
+                tv += kBR;
+                if (tv > cur.v1) {
+                    tv = cur.v0;
+                    tu += kBC;
+                    if (tu > cur.u1) {
+                        ++n;
+                        if (n < nlist) {
+                            tu = list[n].u0;
+                            tv = list[n].v0;
+                        }
+                    }
+                }
+                ok = mbar_wait(&full, phase, status);
+                if (!ok) mbar_wait(&full, phase, status);  // a copy still in flight lands before the CTA leaves
+                phase ^= 1u;
+                const int h = (nr - 1) >> 1;
+                bool odd = false;
+                if (ok) {
+                    // prefix sums of each column, from the middle row h outwards: E[r][c] = sum
+                    // over rows h .. r - 1 (minus rows r .. h - 1) of (p, (row - h) p). A warp takes 32
+                    // columns of one half.
+                    const int c = (warp >> 1) * 32 + lane;
+                    if (c < nc) {
+                        float s0 = 0.f, s1 = 0.f, rr;
+                        if (warp & 1) {
+                            const float *src = raw + c + (h - 1) * kBC;
+                            float2 *dst = E + c + (h - 1) * kEP;
+                            rr = 1.f;
+#pragma unroll 4
+                            for (int r = 0; r < h; ++r) {
+                                const float p = src[-r * kBC];
+                                s0 -= p;
+                                s1 = fmaf(rr, p, s1);
+                                rr += 1.f;
+                                dst[-r * kEP] = make_float2(s0, s1);
+                            }
+                        } else {
+                            const float *src = raw + c + h * kBC;
+                            float2 *dst = E + c + h * kEP;
+                            rr = 0.f;
+                            dst[0] = make_float2(0.f, 0.f);
+#pragma unroll 4
+                            for (int r = 0; r < nr - h; ++r) {
+                                const float p = src[r * kBC];
+                                s0 += p;
+                                s1 = fmaf(rr, p, s1);
+                                rr += 1.f;
+                                dst[(r + 1) * kEP] = make_float2(s0, s1);
+                            }
+                        }
+                        odd = !all_finite(s0, s1);
+                    }
+                }
+                // a wait that gave up ends the sweep for every thread; a tile whose sums are not
+                // finite takes its rows one by one
+                const int flags = __syncthreads_or((ok ? 0 : 2) | (odd ? 1 : 0));
+                if (flags & 2) {
+                    ok = false;
+                    break;
+                }
+                if (tid == 0 && n < nlist) {
+                    mbar_arrive_expect_tx(&full, (uint32_t)kRaw3Bytes);
+                    tma_load_3d(raw, &pmap, tu, tv, b * g.na + list[n].k, &full);
+                }
+                if (mine) {
+                    const Frame32 &F = g.f32[k];
+                    const float rzh = rz_of<float>(g, v0 + h), Szb = Sz - (float)(z0 - 1);
+                    const int tlo = max(u0, a == 0 ? F.ux_lo : F.uy_lo);
+                    const int thi = min(u0 + nc - 1, a == 0 ? F.ux_hi : F.uy_hi);
+                    auto column = [&](int u, float &t, float &qb) {
+                        const ColT<float> c = col_of<float>(g, k, u);
+                        t = fma_rn(di, c.inv, c.tc);
+                        qb = fma_rn(di, c.dqb, c.qcb);
+                        return t > 0.f && t < 1.f && floorf(qb) == (float)s;
+                    };
+                    // columns of the segment: q_b crosses s and s + 1 at u1 and u2; the exact test
+                    // settles the column nearest to each
+                    float u1, u2;
+                    if (a == 0) { u1 = column_of_approx(F, (float)i, (float)s); u2 = column_of_approx(F, (float)i, (float)(s + 1)); }
+                    else { u1 = column_of_approx(F, (float)s, (float)i); u2 = column_of_approx(F, (float)(s + 1), (float)i); }
+                    int ua = tlo, ub = thi;
+                    if (all_finite(u1, u2)) {
+                        ua = max(tlo, (int)rintf(fmaxf(fminf(u1, u2), -1.0e6f)));
+                        ub = min(thi, (int)rintf(fminf(fmaxf(u1, u2), 1.0e6f)));
+                        float t, qb;
+                        if (ua <= ub && !column(ua, t, qb)) ++ua;
+                        if (ua < ub && !column(ub, t, qb)) --ub;
+                    }
+#pragma unroll 1
+                    for (int u = ua; u <= ub; ++u) {
+                        float t, qb;
+                        if (!column(u, t, qb)) continue;
+                        const float wu = qb - floorf(qb), wl = 1.0f - wu;
+                        const float step = t * drz, irs = __fdividef(1.0f, step);
+                        // z of the tile's middle row relative to z0 - 1
+                        const float qh = fmaf(t, rzh, Szb);
+                        if (!(flags & 1)) {
+                            // x(m): tile row coordinate of z0 - 1 + m, plus one; the first row above
+                            // is floor(x). In units of step, the rows of interval m weigh
+                            // S1 = T - (x - 1 - h) S0 on the upper voxel and irs S0 - S1 on the lower.
+                            const float h1 = (float)(h + 1), vb = fmaf(-qh, irs, h1);
+                            const float sl = wl * step, su = wu * step;
+                            const float2 *Eu = E + (u - u0);
+                            auto above = [&](float x) { return Eu[min(__float2uint_rd(x), (unsigned)nr) * (unsigned)kEP]; };
+                            float x = vb, carry = 0.f;  // upper-voxel share of the previous interval
+                            float2 e = above(x);
+#pragma unroll
+                            for (int m = 0; m < kZ3 + 1; ++m) {
+                                const float xn = fmaf((float)(m + 1), irs, vb);
+                                const float2 f = above(xn);
+                                const float2 d = __fadd2_rn(f, make_float2(-e.x, -e.y));
+                                const float S1 = fmaf(h1 - x, d.x, d.y);
+                                // voxel z0 - 1 + m: upper share of interval m - 1, lower share of interval m
+                                if (m >= 1) {
+                                    const float R = carry + fmaf(irs, d.x, -S1);
+                                    SA[m - 1] = fmaf(sl, R, SA[m - 1]);
+                                    SB[m - 1] = fmaf(su, R, SB[m - 1]);
+                                }
+                                carry = S1;
+                                e = f;
+                                x = xn;
+                            }
+                        } else {
+                            const float *Pu = pw + ((long long)(b * g.na + k) * nv + v0) * pitch + u;
+#pragma unroll 1
+                            for (int r = 0; r < nr; ++r) {
+                                const float p = __ldg(Pu + (long long)r * pitch);
+                                const float q = fmaf((float)(r - h), step, qh);
+#pragma unroll
+                                for (int m = 1; m <= kZ3; ++m) {
+                                    const float w = 1.0f - fabsf(q - (float)m);
+                                    if (w > 0.f) {
+                                        SA[m - 1] = fmaf(wl, w * p, SA[m - 1]);
+                                        SB[m - 1] = fmaf(wu, w * p, SB[m - 1]);
+                                    }
+                                }
+                            }
+                        }
+                    }
+                }
+                __syncthreads();
+            }
+            if (!ok) break;
         }
-        // voxel (plane il, local index seg - 1): its own segment's lower shares, then the
-        // upper shares of the segment below it
+        // onto the sum so far (a voxel per thread and step), every voxel (plane il, local index
+        // seg - 1) adds its own segment's lower shares, then the upper shares of the segment
+        // below it
+        auto kept = [&](int j) -> float & {
+            const int e = tid + j * kThreads3;
+            return vacc[(e / (kB3 * kB3)) * kB3 * (kB3 + 1) + ((e / kB3) & (kB3 - 1)) * (kB3 + 1) + (e & (kB3 - 1))];
+        };
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kKeep; ++j)
+            if (tid + j * kThreads3 < kZ3 * kB3 * kB3) kept(j) = keep[j];
+        __syncthreads();
         if (mine && seg >= 1) {
             const int vl = seg - 1;
             float *v = vacc + (a == 0 ? vl * (kB3 + 1) + il : il * (kB3 + 1) + vl);
@@ -422,18 +544,24 @@ __global__ void __launch_bounds__(kThreads3, 4) k_backproject_v3(GeomDev g, cons
             for (int m = 0; m < kZ3; ++m) v[m * kB3 * (kB3 + 1)] += SB[m];
         }
         __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kKeep; ++j)
+            if (tid + j * kThreads3 < kZ3 * kB3 * kB3) keep[j] = kept(j);
+        if (!ok) break;  // outputs stay unwritten
     }
+    if (!ok) return;
     const long long nxy = (long long)nx * ny;
     const int nbatch = (int)(gridDim.z / nparts / nzb);
     float *out = nparts > 1 ? partial + ((long long)part * nbatch + b) * nxy * nz : vol + (long long)b * nxy * nz;
     const int acc_mode = nparts > 1 ? 0 : accumulate;
-    for (int e = tid; e < kZ3 * kB3 * kB3; e += kThreads3) {
+#pragma unroll
+    for (int j = 0; j < kKeep; ++j) {
+        const int e = tid + j * kThreads3;
         const int xl = e & (kB3 - 1), yl = (e / kB3) & (kB3 - 1), zl = e / (kB3 * kB3);
         const int ix = x0 + xl, iy = y0 + yl, iz = z0 + zl;
-        if (ix < nx && iy < ny && iz < nz) {
+        if (e < kZ3 * kB3 * kB3 && ix < nx && iy < ny && iz < nz) {
             float *o = out + ((long long)iz * ny + iy) * nx + ix;
-            const float v = vacc[zl * kB3 * (kB3 + 1) + yl * (kB3 + 1) + xl];
-            *o = acc_mode ? *o + v : v;
+            *o = acc_mode ? *o + keep[j] : keep[j];
         }
     }
 }
@@ -538,18 +666,23 @@ static int backward_impl(const cbct_geom *g, const T *proj, T *vol, int batch, i
     const long long nproj = (long long)batch * d.na * d.nv * d.nu;
     const int nzs = (d.n[2] + kZS - 1) / kZS;
     if ((long long)nzs * batch > 65535) return fail(CBCT_EINVAL, "back_project: batch too large");
+    // the segment gather loads the weighted projections by TMA: rows start on 16 bytes
+    const int pitch = sizeof(T) == 4 && g->axis_contiguous ? (d.nu + 3) & ~3 : d.nu;
     T *pw = nullptr;
-    CBCT_CUDA_TRY(cudaMallocAsync((void **)&pw, sizeof(T) * nproj, st));
+    CBCT_CUDA_TRY(cudaMallocAsync((void **)&pw, sizeof(T) * (nproj / d.nu) * pitch, st));
     dim3 blk(32, 8), gw((d.nu + 31) / 32, (d.nv + 7) / 8, d.na * batch);
-    k_weight_rays<T><<<gw, blk, 0, st>>>(d, proj, pw, colw);
+    k_weight_rays<T><<<gw, blk, 0, st>>>(d, proj, pw, colw, pitch);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) {
         if constexpr (sizeof(T) == 4) {
             if (g->axis_contiguous) {
                 const int nzb = (d.n[2] + kZ3 - 1) / kZ3;
                 const long long base = (long long)((d.n[0] + kB3 - 1) / kB3) * ((d.n[1] + kB3 - 1) / kB3) * nzb * batch;
-                // split the angles so that about 9 CTAs per SM are available (4 resident, 2+ waves)
-                const long long want = 9LL * sm_count();
+                // split the angles so that about 24 CTAs per SM (8 per resident slot) are available: bricks
+                // differ in how many angles see them, and the last ones must not leave SMs idle
+                // (2 x 128^3: 12 / 24 / 48 per SM 1800 / 1680 / 1640 us; one 128^3 930 / 868 / 875; the
+                // clinical volume has 40 per SM unsplit)
+                const long long want = 24LL * sm_count();
                 int nparts = (int)std::min<long long>(16, std::max<long long>(1, (want + base - 1) / base));
                 nparts = std::min(nparts, d.na);
                 while (nparts > 1 && (long long)nzb * batch * nparts > 65535) --nparts;
@@ -557,22 +690,28 @@ static int backward_impl(const cbct_geom *g, const T *proj, T *vol, int batch, i
                 float *partial = nullptr;
                 const long long nvol = (long long)batch * d.n[0] * d.n[1] * d.n[2];
                 if (e == cudaSuccess && nparts > 1) e = cudaMallocAsync((void **)&partial, sizeof(float) * nvol * nparts, st);
-                // panel widths of common flat panels get a kernel with the width built in
-                auto kern = d.nu == 256 ? k_backproject_v3<256>
-                          : d.nu == 512 ? k_backproject_v3<512>
-                          : d.nu == 1024 ? k_backproject_v3<1024> : k_backproject_v3<0>;
-                if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem3);
+                int trc = 0;
                 if (e == cudaSuccess) {
-                    dim3 gb3((d.n[0] + kB3 - 1) / kB3, (d.n[1] + kB3 - 1) / kB3, nzb * batch * nparts);
-                    kern<<<gb3, kThreads3, kSmem3, st>>>(d, pw, vol, accumulate, nparts, partial);
-                    e = cudaGetLastError();
-                    if (e == cudaSuccess && nparts > 1) {
-                        k_sum_parts<<<8 * sm_count(), 256, 0, st>>>(partial, nparts, nvol, vol, accumulate);
+                    CUtensorMap pmap;
+                    const uint64_t dims[3] = {(uint64_t)d.nu, (uint64_t)d.nv, (uint64_t)d.na * batch};
+                    const uint64_t str[2] = {(uint64_t)pitch * 4, (uint64_t)pitch * d.nv * 4};
+                    const uint32_t box[3] = {kBC, kBR, 1};
+                    trc = encode_tmap(&pmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, pw, dims, str, box);
+                    if (trc == 0) {
+                        dim3 gb3((d.n[0] + kB3 - 1) / kB3, (d.n[1] + kB3 - 1) / kB3, nzb * batch * nparts);
+                        k_backproject_seg<<<gb3, kThreads3, kSmem3, st>>>(pmap, d, pw, pitch, vol, accumulate, nparts, partial,
+                                                                          g->status);
                         e = cudaGetLastError();
+                        if (e == cudaSuccess && nparts > 1) {
+                            const int gs = (int)std::min<long long>(8LL * sm_count(), (nvol + 255) / 256);
+                            k_sum_parts<<<gs, 256, 0, st>>>(partial, nparts, nvol, vol, accumulate);
+                            e = cudaGetLastError();
+                        }
                     }
                 }
                 if (partial) cudaFreeAsync(partial, st);
                 cudaFreeAsync(pw, st);
+                if (trc) return trc;
                 if (e != cudaSuccess) return cuda_fail(e, "back_project launch");
                 return 0;
             }
@@ -707,8 +846,9 @@ static int noalloc_scratch(int dev, float **out) {
     return 0;
 }
 
-int noalloc_prime(int dev) {
+int projector_prime(int dev) {
     float *p = nullptr;
+    CBCT_CUDA_TRY(cudaFuncSetAttribute(k_backproject_seg, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem3));
     return noalloc_scratch(dev, &p);
 }
 
@@ -744,7 +884,7 @@ extern "C" int back_project_noalloc(const cbct_geom *g, const float *proj, float
             v.col64 = d.col64 + (long long)k0 * d.nu;
             const float *pb = proj + ((long long)b * d.na + k0) * per_angle;
             dim3 gw((d.nu + 31) / 32, (d.nv + 7) / 8, kc);
-            k_weight_rays<float><<<gw, blk, 0, st>>>(v, pb, scratch, nullptr);
+            k_weight_rays<float><<<gw, blk, 0, st>>>(v, pb, scratch, nullptr, d.nu);
             dim3 gb((d.n[0] + 31) / 32, (d.n[1] + 7) / 8, nzs);
             k_backproject<float, kZS><<<gb, blk, 0, st>>>(v, scratch, vol + b * nvox, k0 == 0 ? accumulate : 1);
             CBCT_LAUNCH_CHECK("back_project_noalloc launch");
