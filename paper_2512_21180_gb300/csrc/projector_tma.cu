@@ -350,7 +350,8 @@ __global__ void __launch_bounds__(kThreads) k_forward_tma(const __grid_constant_
             const bool ray_ok = col_ok && iv < g.nv;
             const float r = ray_ok ? (rr ? acc.y * step.y : acc.x * step.x) * g.scale : 0.f;
             float *out = proj + (((long long)b * g.na + k) * g.nv + iv) * g.nu + iu;
-            if ((g.nu & 3) == 0 && u0 + kTU <= g.nu && iv < g.nv) {  // uniform over the warp
+            if ((g.nu & 3) == 0 && (reinterpret_cast<uintptr_t>(proj) & 15) == 0 && u0 + kTU <= g.nu &&
+                iv < g.nv) {  // uniform over the warp
                 const float r1 = __shfl_down_sync(0xffffffffu, r, 1);
                 const float r2 = __shfl_down_sync(0xffffffffu, r, 2);
                 const float r3 = __shfl_down_sync(0xffffffffu, r, 3);

@@ -22,6 +22,10 @@ static int grid1(long long n) {
     return (int)std::max<long long>(1, std::min<long long>(b, 32LL * sm_count()));
 }
 
+// Floats of a scratch array rounded up so that the next one starts on 256 bytes: the projector
+// reads and writes whole 16-byte groups where its buffers allow it.
+static long long padded(long long n) { return (n + 63) & ~63LL; }
+
 // ---- FDK ---------------------------------------------------------------------------
 
 // q0[b][k][v][e] = proj * w(u) * sdd / sqrt(sdd^2 + u^2 + v^2) on the extended row
@@ -324,10 +328,10 @@ extern "C" int cbct_opnorm(const cbct_geom *g, double gamma, int iters, double *
     const long long nvox = (long long)d.n[0] * d.n[1] * d.n[2], nproj = (long long)d.na * d.nv * d.nu;
     float *x = nullptr, *p = nullptr, *y = nullptr;
     double *acc = nullptr;
-    CBCT_CUDA_TRY(cudaMallocAsync((void **)&x, sizeof(float) * (2 * nvox + nproj) + 16, st));
-    y = x + nvox;
-    p = y + nvox;
-    acc = reinterpret_cast<double *>(p + nproj + (nproj & 1));
+    CBCT_CUDA_TRY(cudaMallocAsync((void **)&x, sizeof(float) * (2 * padded(nvox) + padded(nproj)) + 16, st));
+    y = x + padded(nvox);
+    p = y + padded(nvox);
+    acc = reinterpret_cast<double *>(p + padded(nproj));
     int rc = 0;
     k_fill1<<<grid1(nvox), 256, 0, st>>>(x, nvox, 1.0f);
     double nrm2 = 0.0;
@@ -364,11 +368,12 @@ extern "C" int cbct_pdhg(const cbct_geom *g, const float *y, const float *x0, fl
     const long long N = (long long)batch * d.n[0] * d.n[1] * d.n[2], M = (long long)batch * d.na * d.nv * d.nu;
     float *buf = nullptr;
     // xbar, bt (N each), z2 (3N), z1, p (M each)
-    CBCT_CUDA_TRY(cudaMallocAsync((void **)&buf, sizeof(float) * (5 * N + 2 * M), st));
-    float *xb = buf, *bt = xb + N, *z2 = bt + N, *z1 = z2 + 3 * N, *p = z1 + M;
+    const long long Np = padded(N), Mp = padded(M), N3 = padded(3 * N);
+    CBCT_CUDA_TRY(cudaMallocAsync((void **)&buf, sizeof(float) * (2 * Np + N3 + 2 * Mp), st));
+    float *xb = buf, *bt = xb + Np, *z2 = bt + Np, *z1 = z2 + N3, *p = z1 + Mp;
     if (x != x0) cudaMemcpyAsync(x, x0, sizeof(float) * N, cudaMemcpyDeviceToDevice, st);
     cudaMemcpyAsync(xb, x0, sizeof(float) * N, cudaMemcpyDeviceToDevice, st);
-    cudaMemsetAsync(z2, 0, sizeof(float) * (3 * N + M), st);
+    cudaMemsetAsync(z2, 0, sizeof(float) * (N3 + M), st);
     int rc = 0;
     const float rad = (float)(lam / gamma);
     for (int it = 0; it < niter && rc == 0; ++it) {
@@ -395,8 +400,8 @@ extern "C" int cbct_landweber(const cbct_geom *g, const float *y, float *x, int 
     const GeomDev &d = g->dev;
     const long long N = (long long)batch * d.n[0] * d.n[1] * d.n[2], M = (long long)batch * d.na * d.nv * d.nu;
     float *buf = nullptr;
-    CBCT_CUDA_TRY(cudaMallocAsync((void **)&buf, sizeof(float) * (N + M), st));
-    float *gr = buf, *r = buf + N;
+    CBCT_CUDA_TRY(cudaMallocAsync((void **)&buf, sizeof(float) * (padded(N) + M), st));
+    float *gr = buf, *r = buf + padded(N);
     int rc = 0;
     for (int it = 0; it < niter && rc == 0; ++it) {
         rc = forward_project(g, x, r, batch, 0, stream);
