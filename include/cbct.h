@@ -107,16 +107,17 @@ double geometry_scale(const cbct_geom *g);
 int cbct_device_status(const cbct_geom *g, int *out, int clear);
 
 /* Staged-forward configuration chosen for this geometry: *cfg = index of the
- * shared-memory box (0..3) or -1 for the direct kernel; *need_b / *need_z = host
- * bounds of a 32 x 8 ray tile's footprint over 8 planes (voxels). Any pointer may
- * be NULL. */
+ * shared-memory box (0..6, smallest first) or -1 for the direct kernel; *need_b /
+ * *need_z = host bounds of a 32 x 16 ray tile's footprint over 8 planes (voxels). Any
+ * pointer may be NULL. */
 int cbct_forward_config(const cbct_geom *g, int *cfg, double *need_b, double *need_z);
 
 /* Forward projection (a2, Sec. 2.2): proj[b] (+)= P vol[b] for b < batch.
  * accumulate = 0 overwrites proj, 1 adds to it. FP32 in, FP32 accumulation.
- * batch >= 1; batch * n_angles <= 65535. Scratch: two plane-major copies of the
- * volumes (2 * batch * nx * ny * nz floats, rows padded to 4), from the
- * stream-ordered pool. Errors: CBCT_EINVAL (before any launch) for a NULL pointer,
+ * batch >= 1; batch * n_angles <= 65535. Scratch: a plane-major copy of the
+ * volumes (batch * nx * ny * nz floats, rows padded to 4; a second one when nx is not a
+ * multiple of 4 or vol not on 16 bytes), from the stream-ordered pool; none for calls of
+ * at most 2^20 rays times planes. Errors: CBCT_EINVAL (before any launch) for a NULL pointer,
  * batch < 1, accumulate not 0 or 1, batch * n_angles > 65535 or a current device
  * other than the geometry's; CBCT_ENOMEM when the scratch cannot be allocated;
  * CBCT_ECUDA for a failed launch. */

@@ -67,7 +67,9 @@ int conv_pack_jobs(const ConvPackJob *jobs, int njobs, long long max_nelem, cons
 // back_project_noalloc's fixed scratch array, so that the module holding the array is
 // loaded, and the array placed, when the geometry is made.
 int projector_prime(int dev);
+// Ray tile of the staged forward (columns x rows).
+constexpr int kForwardTileCols = 32, kForwardTileRows = 16;
 // Staged (TMA) forward: returns 1 if it ran, 0 if the direct kernel must be used.
 int forward_staged(const cbct_geom *g, const float *vol, float *proj, int batch, int accumulate, cudaStream_t st);
-int choose_forward_cfg(double need_b, double need_z);
+int choose_forward_cfg(double need_b, double need_z, double slope_b, double slope_z);
 }  // namespace cbct

@@ -135,14 +135,15 @@ static void build_columns(const cbct_geom_desc &d, const std::vector<Frame32> &f
     }
 }
 
-// Bounds on the footprint of a 32 x 8 ray tile over one 8-plane chunk (the staged
-// forward's TMA box must hold it): per-column changes of the central-plane
-// parameters times the tile width, plane slopes times the chunk depth, plus
-// neighbour, floor and alignment margins. Also checks that at every angle the
+// Bounds on the footprint of a 32 x 16 ray tile on one plane (need), and per further plane
+// of a chunk (slope): the staged forward's TMA box must hold it. Per-column changes of
+// the central-plane parameters times the tile width, plus neighbour, floor and
+// alignment margins. Also checks that at every angle the
 // x- and y-principal columns form intervals.
 static void forward_bounds(const cbct_geom_desc &d, const std::vector<Frame32> &f32, const std::vector<Col64> &c64,
-                           const std::vector<double> &rz64, double &need_b, double &need_z, bool &contiguous) {
-    const int TU = 32, TV = 8, P = 8;
+                           const std::vector<double> &rz64, double &need_b, double &need_z, double &slope_b,
+                           double &slope_z, bool &contiguous) {
+    const int TU = cbct::kForwardTileCols, TV = cbct::kForwardTileRows;
     const int n[2] = {d.nx, d.ny};
     double rzmax = 0.0;
     for (double r : rz64) rzmax = std::max(rzmax, std::fabs(r));
@@ -169,8 +170,11 @@ static void forward_bounds(const cbct_geom_desc &d, const std::vector<Frame32> &
             }
         }
     }
-    need_b = (TU - 1) * Mb + (P - 1) * Dq + 8.0;
-    need_z = (TV - 1) * tmax * drz + (TU - 1) * Mzu + (P - 1) * Dz + 5.0;
+    need_b = (TU - 1) * Mb + 8.0;
+    slope_b = Dq;
+    slope_z = Dz;
+    // four rows of a thread span ceil(3 tmax drz) + 1 cells, and it reads that many levels
+    need_z = (TV - 1) * tmax * drz + (TU - 1) * Mzu + 5.0 + ceil(3.0 * tmax * drz * 1.0001 + 1e-4);
 }
 
 // No ray may have z as its principal axis: at every angle the smallest
@@ -226,8 +230,11 @@ extern "C" int geometry_create(const cbct_geom_desc *desc, cbct_geom **out) {
     std::vector<double> rz64;
     build_columns(d, f32, f64, c32, c64, rz32, rz64);
     const size_t ncol = (size_t)d.n_angles * d.nu;
-    forward_bounds(d, f32, c64, rz64, g->fwd_need_b, g->fwd_need_z, g->axis_contiguous);
-    g->fwd_cfg = g->axis_contiguous ? choose_forward_cfg(g->fwd_need_b, g->fwd_need_z) : -1;
+    double slope_b = 0.0, slope_z = 0.0;
+    forward_bounds(d, f32, c64, rz64, g->fwd_need_b, g->fwd_need_z, slope_b, slope_z, g->axis_contiguous);
+    g->fwd_cfg = g->axis_contiguous ? choose_forward_cfg(g->fwd_need_b, g->fwd_need_z, slope_b, slope_z) : -1;
+    g->fwd_need_b += 7 * slope_b;  // reported for eight planes
+    g->fwd_need_z += 7 * slope_z;
     e = cudaMalloc(&g->status, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(g->status, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&g->f32, sizeof(Frame32) * d.n_angles);

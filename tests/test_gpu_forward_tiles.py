@@ -1,0 +1,88 @@
+"""Staged forward projection at the edges of its tiling: every box configuration, rows that span
+two and more z-cells, rows and columns past the panel, volumes whose rows do not start on 16
+bytes, planes cut by the panel, small calls on the direct kernel, and non-finite voxels. The
+reference is the FP64 instantiation, an independent kernel with one thread per ray."""
+import ctypes
+
+import pytest
+import torch
+
+from paper_2512_21180_gb300 import _lib
+from paper_2512_21180_gb300 import inputs as I
+from paper_2512_21180_gb300 import projector as P
+
+pytestmark = pytest.mark.gpu
+
+T = I.geometry("tiny16")
+
+
+def scan(n, vox, nu, nv, du, dv, na=9, **kw):
+    return I.scaled(T, n=n, vox=(vox, vox, 4.0 if vox > 2 else 2.0), nu=nu, nv=nv, du=du, dv=dv, n_angles=na, **kw)
+
+
+# name -> (geometry, box configuration chosen for it)
+CASES = {
+    "box0": (scan((64, 60, 40), 4.0, 130, 70, 1.2, 1.2), 0),
+    "box1_ragged": (scan((61, 63, 41), 4.0, 121, 50, 1.6, 1.6, u_offset=30.0, v_offset=5.0), 1),
+    "box2": (scan((60, 64, 40), 4.0, 101, 45, 2.4, 2.7), 2),
+    "box3": (scan((60, 66, 40), 4.0, 81, 45, 3.2, 3.4), 3),
+    "box5_four_cells": (scan((67, 64, 40), 4.0, 61, 33, 4.5, 5.0, 15), 5),
+    "box6_five_cells": (scan((67, 64, 40), 2.5, 61, 33, 4.5, 6.0, 15), 6),
+    "direct": (scan((64, 64, 40), 2.0, 61, 33, 7.0, 7.0, 15), -1),
+    "panel_cuts_volume": (scan((96, 96, 24), 12.0, 150, 40, 4.0, 4.0, 15), 5),
+    "nv_one": (scan((64, 60, 40), 4.0, 1030, 1, 0.4, 1.2, 20), None),
+}
+TOL = 1e-5  # the FP32 projector pair's bar against 64 bits
+
+
+def check(got, ref):
+    assert float((got.double() - ref).norm()) <= TOL * float(ref.norm())
+    assert float((got.double() - ref).abs().max()) <= TOL * float(ref.abs().max())
+
+
+@pytest.mark.parametrize("batch", [1, 2])
+@pytest.mark.parametrize("name", list(CASES))
+def test_boxes_match_fp64(name, batch):
+    g, cfg = CASES[name]
+    geom = P.Geometry(g)
+    c = ctypes.c_int()
+    _lib.check(_lib.load().cbct_forward_config(geom.handle, ctypes.byref(c), None, None))
+    assert cfg is None or c.value == cfg
+    x = torch.as_tensor(I.random_volume((batch,) + geom.vol_shape, 17), device="cuda")
+    got = P.forward_project(geom, x)
+    check(got, P.forward_project(geom, x.double()))
+    acc = P.forward_project(geom, x, out=torch.ones_like(got), accumulate=True)
+    assert float((acc - 1.0 - got).abs().max()) <= 4e-7 * (1.0 + float(got.abs().max()))
+    assert torch.equal(got, P.forward_project(geom, x))
+    assert geom.device_status() == 0
+
+
+def test_volume_rows_off_16_bytes():
+    """A contiguous volume at an odd element offset of a larger buffer (x rows of 64 voxels)."""
+    geom = P.Geometry(CASES["box0"][0])
+    n = 64 * 60 * 40
+    buf = torch.as_tensor(I.random_volume((n + 3,), 4), device="cuda")
+    want = P.forward_project(geom, buf[3:].clone().reshape((1,) + geom.vol_shape))
+    assert torch.equal(P.forward_project(geom, buf[3:].reshape((1,) + geom.vol_shape)), want)
+
+
+@pytest.mark.parametrize("name", ["box0", "box1_ragged", "box5_four_cells", "panel_cuts_volume"])
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), float("-inf")])
+def test_non_finite_voxels_reach_only_their_rays(name, value):
+    """The rays whose bilinear footprint holds the voxel (the FP64 projection of that voxel alone)
+    become non-finite, every other ray keeps its value."""
+    geom = P.Geometry(CASES[name][0])
+    x = torch.as_tensor(I.random_volume((1,) + geom.vol_shape, 8), device="cuda")
+    clean = P.forward_project(geom, x)
+    at = (0,) + tuple(n // 2 for n in geom.vol_shape)
+    one = torch.zeros_like(x, dtype=torch.float64)
+    one[at] = 1.0
+    w = P.forward_project(geom, one)
+    x[at] = value
+    got = P.forward_project(geom, x)
+    touched = w > 1e-4 * w.max()
+    assert int(touched.sum()) >= 9
+    assert not bool(torch.isfinite(got[touched]).any())
+    far = w == 0
+    assert bool(torch.isfinite(got[far]).all())
+    assert float((got[far] - clean[far]).abs().max()) <= TOL * float(clean.abs().max())
