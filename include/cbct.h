@@ -187,7 +187,8 @@ int cbct_phantom(const cbct_geom *g, const double *ell_host, int n_ell, int supe
  * Poisson(I0 exp(-line_integrals[e])) for e < n, device arrays. Random words come
  * from Philox4x32-10 (Salmon et al., SC'11) with key (seed lo, seed hi) and counter
  * (e lo, e hi, block, 0x50303031); means below 10 are sampled by inversion, others
- * by Hoermann's PTRS (1993); decisions in FP64. Deterministic for a given seed. */
+ * by Hoermann's PTRS (1993); the counts are those of FP64 decisions. Deterministic for a
+ * given seed. */
 int cbct_poisson(const float *line_integrals, long long n, double I0, unsigned long long seed, int32_t *counts,
                  void *stream);
 

@@ -18,6 +18,7 @@
 
 #include "common.cuh"
 #include "geom_impl.h"
+#include "poisson.cuh"
 
 namespace cbct {
 
@@ -69,70 +70,19 @@ __global__ void k_phantom(GeomDev g, const double *__restrict__ ell, int nell, i
     }
 }
 
-// ---- Philox4x32-10 and Poisson -----------------------------------------------------
+// ---- Poisson counts (poisson.cuh) ------------------------------------------------------
 
-__device__ __forceinline__ uint4 philox(uint4 c, uint32_t k0, uint32_t k1) {
-#pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        if (r) { k0 += 0x9E3779B9u; k1 += 0xBB67AE85u; }
-        const uint32_t hi0 = __umulhi(0xD2511F53u, c.x), lo0 = 0xD2511F53u * c.x;
-        const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z), lo1 = 0xCD9E8D57u * c.z;
-        c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
-    }
-    return c;
-}
-
-__device__ __forceinline__ double u01(uint32_t x) { return ((double)x + 0.5) * (1.0 / 4294967296.0); }
-
-// One Poisson(lam) draw for element e: key (seed lo, seed hi), counter
-// (e lo, e hi, block, 0x50303031); block 0 word 0 for inversion (lam < 10); blocks
-// 0, 1, ... two words per attempt for PTRS (lam >= 10).
-__device__ int32_t poisson_draw(double lam, unsigned long long e, unsigned long long seed) {
-    if (!(lam > 0.0)) return 0;
-    const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-    uint4 ctr = make_uint4((uint32_t)e, (uint32_t)(e >> 32), 0u, 0x50303031u);
-    // every step rounded as written (no FMA contraction), as in the definition
-    if (lam < 10.0) {
-        const uint4 r = philox(ctr, k0, k1);
-        const double u = u01(r.x);
-        double p = exp(-lam), F = p;
-        int32_t k = 0;
-        while (u > F && k < 1000) {
-            k++;
-            p = __dmul_rn(p, __ddiv_rn(lam, (double)k));
-            F = __dadd_rn(F, p);
-        }
-        return k;
-    }
-    const double slam = sqrt(lam), loglam = log(lam);
-    const double b = __dadd_rn(0.931, __dmul_rn(2.53, slam));
-    const double a = __dadd_rn(-0.059, __dmul_rn(0.02483, b));
-    const double inv_alpha = __dadd_rn(1.1239, __ddiv_rn(1.1328, __dsub_rn(b, 3.4)));
-    const double vr = __dsub_rn(0.9277, __ddiv_rn(3.6224, __dsub_rn(b, 2.0)));
-    const double twoa = __dmul_rn(2.0, a);
-    for (uint32_t j = 0; j < 4096u; ++j) {
-        ctr.z = j;
-        const uint4 r = philox(ctr, k0, k1);
-        const uint32_t w[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const double U = __dsub_rn(u01(w[2 * h]), 0.5), V = u01(w[2 * h + 1]);
-            const double us = __dsub_rn(0.5, fabs(U));
-            const double kf = floor(__dadd_rn(__dadd_rn(__dmul_rn(__dadd_rn(__ddiv_rn(twoa, us), b), U), lam), 0.43));
-            if (us >= 0.07 && V <= vr) return (int32_t)kf;
-            if (kf < 0.0 || (us < 0.013 && V > us)) continue;
-            const double lhs = log(__ddiv_rn(__dmul_rn(V, inv_alpha), __dadd_rn(__ddiv_rn(a, __dmul_rn(us, us)), b)));
-            const double rhs = __dsub_rn(__dadd_rn(-lam, __dmul_rn(kf, loglam)), lgamma(__dadd_rn(kf, 1.0)));
-            if (lhs <= rhs) return (int32_t)kf;
-        }
-    }
-    return (int32_t)floor(lam + 0.5);
+// One count of mean I0 exp(-p); I0 = ih + il.
+__device__ __forceinline__ int32_t poisson_count(float p, double I0, float ih, float il, unsigned long long e,
+                                                 unsigned long long seed) {
+    const int32_t c = poisson_fast(mean32(ih, il, p, 0.f), e, seed);
+    return c >= 0 ? c : poisson_draw(__dmul_rn(I0, exp(-(double)p)), e, seed);
 }
 
 __global__ void k_poisson(const float *__restrict__ p, long long n, double I0, unsigned long long seed,
                           int32_t *__restrict__ counts) {
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
-        counts[e] = poisson_draw(__dmul_rn(I0, exp(-(double)p[e])), (unsigned long long)e, seed);
+        counts[e] = poisson_count(p[e], I0, (float)I0, (float)(I0 - (double)(float)I0), (unsigned long long)e, seed);
 }
 
 __global__ void k_neglog(const int32_t *__restrict__ counts, long long n, float I0, float *__restrict__ y) {
@@ -147,7 +97,7 @@ __global__ void k_poisson_neglog(const float *__restrict__ p, long long n, doubl
                                  float *__restrict__ y) {
     const float I0f = (float)I0;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        const int32_t N = poisson_draw(__dmul_rn(I0, exp(-(double)p[e])), (unsigned long long)e, seed);
+        const int32_t N = poisson_count(p[e], I0, I0f, (float)(I0 - (double)I0f), (unsigned long long)e, seed);
         const float c = N < 1 ? 1.0f : (float)N;
         y[e] = -logf(fminf(c / I0f, 1.0f));
     }
@@ -160,6 +110,7 @@ constexpr int kPolyMaxBins = 16;
 struct PolyTab {
     int ne;
     double muw[kPolyMaxBins], mub[kPolyMaxBins], resp[kPolyMaxBins];
+    float muw32[kPolyMaxBins][2], mub32[kPolyMaxBins][2];  // the attenuations as hi + lo
     double rmin;  // smallest resp_j: the reading of one photon in the least responsive bin
 };
 
@@ -196,28 +147,48 @@ __global__ void k_water_bone(const float *__restrict__ mu, long long nvox, long 
 // Poisson(lam_j) drawn on the counter of element e ne + j (lam_j itself when noise
 // is 0); y = -log(min(max(reading, rmin) / air, 1)) with the expected air reading
 // air = sum_j resp_j I0[j][pix] (a reading of zero photons is taken as one photon of
-// the least responsive bin, as the monochromatic path clamps counts to one). FP64
-// throughout, each operation rounded as written.
-__global__ void k_poly_reading(const float *__restrict__ L, long long per_item, long long n, int npix,
-                               const float *__restrict__ I0, PolyTab t, unsigned long long seed, int noise,
-                               float *__restrict__ reading, float *__restrict__ y, int32_t *__restrict__ counts) {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        const long long b = e / per_item, r = e - b * per_item;
-        const int pix = (int)(r % npix);
-        const double Lw = (double)L[(2 * b) * per_item + r], Lb = (double)L[(2 * b + 1) * per_item + r];
-        double acc = 0.0, air = 0.0;
+// the least responsive bin, as the monochromatic path clamps counts to one). Readings and
+// logarithms in FP64, each operation rounded as written.
+//
+// A thread takes one pixel in `group` frames (views of all items), so the air reading is summed
+// once. With FP64 draws the kernel was bound by the FP64 pipe (83 % of it); the draws of
+// poisson.cuh decide all but 1e-4 of them in FP32. 9.8 M pixels x 10 bins (CUDA events): 66.7 ms ->
+// 2.4 ms (41 G draws/s).
+__global__ void __launch_bounds__(256) k_poly_reading(const float *__restrict__ L, int frames_per_item, int nframes,
+                                                      int npix, int group, const float *__restrict__ I0, PolyTab t,
+                                                      unsigned long long seed, int noise, float *__restrict__ reading,
+                                                      float *__restrict__ y, int32_t *__restrict__ counts) {
+    const int pix = blockIdx.x * blockDim.x + threadIdx.x;
+    if (pix >= npix) return;
+    const int f0 = blockIdx.y * group, f1 = min(f0 + group, nframes);
+    double air = 0.0;
+    for (int j = 0; j < t.ne; ++j) air = __dadd_rn(air, __dmul_rn(t.resp[j], (double)I0[(long long)j * npix + pix]));
+    const long long per_item = (long long)frames_per_item * npix;
+    for (int f = f0; f < f1; ++f) {
+        const int b = f / frames_per_item;
+        const long long e = (long long)f * npix + pix, w = e + b * per_item;  // water; bone one item on
+        const float Lw = L[w], Lb = L[w + per_item];
+        double acc = 0.0;
         for (int j = 0; j < t.ne; ++j) {
-            const double i0 = (double)I0[(long long)j * npix + pix];
-            const double a = __dadd_rn(__dmul_rn(t.muw[j], Lw), __dmul_rn(t.mub[j], Lb));
-            const double lam = __dmul_rn(i0, exp(-a));
-            double v = lam;
+            const float i0 = I0[(long long)j * npix + pix];
+            double v;
+            auto mean = [&]() {
+                return __dmul_rn((double)i0, exp(-__dadd_rn(__dmul_rn(t.muw[j], (double)Lw), __dmul_rn(t.mub[j], (double)Lb))));
+            };
             if (noise) {
-                const int32_t c = poisson_draw(lam, (unsigned long long)e * (unsigned long long)t.ne + j, seed);
+                // mu_w L_w + mu_b L_b as hi + lo: both products and their sum with their roundings
+                const float p = t.muw32[j][0] * Lw, q = t.mub32[j][0] * Lb, a = p + q, z = a - p;
+                const float alo = (fmaf(t.muw32[j][0], Lw, -p) + t.muw32[j][1] * Lw) +
+                                  (fmaf(t.mub32[j][0], Lb, -q) + t.mub32[j][1] * Lb) + ((p - (a - z)) + (q - z));
+                const unsigned long long ej = (unsigned long long)e * (unsigned long long)t.ne + j;
+                int32_t c = i0 == 0.f ? 0 : poisson_fast(mean32(i0, 0.f, a, alo), ej, seed);
+                if (c < 0) c = poisson_draw(mean(), ej, seed);
                 if (counts) counts[e * t.ne + j] = c;
                 v = (double)c;
+            } else {
+                v = mean();
             }
             acc = __dadd_rn(acc, __dmul_rn(t.resp[j], v));
-            air = __dadd_rn(air, __dmul_rn(t.resp[j], i0));
         }
         if (reading) reading[e] = (float)acc;
         if (y) y[e] = (float)(-log(fmin(__ddiv_rn(fmax(acc, t.rmin), air), 1.0)));
@@ -246,6 +217,10 @@ static int poly_table(int n_e, const double *energies, const double *mu_w, const
         t->muw[j] = mu_w[j];
         t->mub[j] = mu_b[j];
         t->resp[j] = detector_response(energies[j]);
+        t->muw32[j][0] = (float)mu_w[j];
+        t->muw32[j][1] = (float)(mu_w[j] - (double)t->muw32[j][0]);
+        t->mub32[j][0] = (float)mu_b[j];
+        t->mub32[j][1] = (float)(mu_b[j] - (double)t->mub32[j][0]);
         t->rmin = fmin(t->rmin, t->resp[j]);
     }
     return 0;
@@ -296,6 +271,22 @@ __global__ void k_fov(GeomDev g, const double *__restrict__ cs, double sid, doub
         }
         V[q] = (float)((double)cnt / g.na);
     }
+}
+
+// Frames per thread of k_poly_reading: enough threads for four waves of 2048 per SM, at most 16
+// frames, and at most 65535 groups.
+static int poly_launch(const float *L, int batch, long long n_per_item, int npix, const float *I0, const PolyTab &t,
+                       unsigned long long seed, int noise, float *reading, float *y, int32_t *counts, cudaStream_t st) {
+    const long long frames_per_item = n_per_item / npix, nframes = frames_per_item * batch;
+    if (nframes > 0x7fffffffLL) return fail(CBCT_EINVAL, "cbct_poly_reading: too many frames");
+    long long group = nframes * npix / (4LL * 2048 * sm_count());
+    group = group < 1 ? 1 : group > 16 ? 16 : group;
+    if ((nframes + group - 1) / group > 65535) group = (nframes + 65534) / 65535;
+    dim3 grd((unsigned)((npix + 255) / 256), (unsigned)((nframes + group - 1) / group));
+    k_poly_reading<<<grd, 256, 0, st>>>(L, (int)frames_per_item, (int)nframes, npix, (int)group, I0, t, seed, noise ? 1 : 0,
+                                        reading, y, counts);
+    CBCT_LAUNCH_CHECK("cbct_poly_reading launch");
+    return 0;
 }
 
 static int grid_for(long long n) {
@@ -424,10 +415,8 @@ extern "C" int cbct_poly_reading(const float *line_integrals, int batch, long lo
         return fail(CBCT_EINVAL, "cbct_poly_reading: invalid argument");
     const long long n = n_per_item * batch;
     if (n == 0) return 0;
-    k_poly_reading<<<grid_for(n), 256, 0, (cudaStream_t)stream>>>(line_integrals, n_per_item, n, npix, I0, t, seed,
-                                                                  noise ? 1 : 0, reading, y, counts);
-    CBCT_LAUNCH_CHECK("cbct_poly_reading launch");
-    return 0;
+    return poly_launch(line_integrals, batch, n_per_item, npix, I0, t, seed, noise, reading, y, counts,
+                       (cudaStream_t)stream);
 }
 
 extern "C" int cbct_poly_simulate(const cbct_geom *g, const float *mu, int batch, double mu_water60, int n_e,
@@ -454,9 +443,5 @@ extern "C" int cbct_poly_simulate(const cbct_geom *g, const float *mu, int batch
     rc = forward_project(g, rho, line_integrals, 2 * batch, 0, stream);
     cudaFreeAsync(rho, st);
     if (rc) return rc;
-    k_poly_reading<<<grid_for(per_item * batch), 256, 0, st>>>(line_integrals, per_item, per_item * batch,
-                                                              v.nv * v.nu, I0, t, seed, noise ? 1 : 0, nullptr, y,
-                                                              nullptr);
-    CBCT_LAUNCH_CHECK("cbct_poly_simulate: reading launch");
-    return 0;
+    return poly_launch(line_integrals, batch, per_item, v.nv * v.nu, I0, t, seed, noise, nullptr, y, nullptr, st);
 }
