@@ -1,0 +1,64 @@
+"""FDK_w over its row filters (direct, transforms of 1024, 2048 and 4096 points) and angle splits,
+against the FP64 oracle: odd row counts (a last row without a partner), batches, accumulation, and
+rows with a non-finite value, which must not reach the rows they share a transform with."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2512_21180_gb300 import _lib
+from paper_2512_21180_gb300 import inputs as I
+from paper_2512_21180_gb300 import ops
+from paper_2512_21180_gb300 import projector as P
+
+from gpu_util import rel_l2, to_gpu, to_np
+
+pytestmark = pytest.mark.gpu
+
+B = I.geometry("small64")
+CASES = {
+    "direct_wide": I.scaled(B, n=(20, 18, 9), nu=2050, nv=3, du=0.2, dv=8.0, n_angles=8),
+    "direct_small_split": I.scaled(B, n=(23, 21, 17), nu=90, nv=31, du=3.0, dv=5.0, n_angles=70, u_offset=30.0),
+    "fft1024": I.scaled(B, n=(24, 26, 19), nu=300, nv=41, du=1.1, dv=4.0, n_angles=30),
+    "fft1024_edge": I.scaled(B, n=(24, 26, 19), nu=512, nv=35, du=0.6, dv=4.0, n_angles=30, v_offset=9.0),
+    "fft2048_offset": I.scaled(B, n=(24, 26, 19), nu=400, nv=37, du=0.9, dv=4.0, n_angles=30, u_offset=-110.0),
+    "fft4096": I.scaled(B, n=(24, 26, 19), nu=1300, nv=35, du=0.25, dv=4.0, n_angles=30, u_offset=60.0),
+}
+
+
+@pytest.mark.parametrize("name", list(CASES))
+def test_paths_match_oracle(O, name):
+    g = CASES[name]
+    G, geom = O.Geom(g), P.Geometry(g)
+    y = np.stack([O.forward(G, O.phantom(G, I.ellipsoids(g, 3 + b, n_soft=6, axes_mm=(8.0, 50.0)))) for b in range(2)])
+    y = y.astype(np.float32)
+    got = ops.fdk(geom, to_gpu(y))
+    for b in range(2):
+        assert rel_l2(to_np(got[b]), O.fdk(G, y[b].astype(np.float64))) <= 1e-4  # the FDK bar (positions in FP32)
+    assert torch.equal(ops.fdk(geom, to_gpu(y)), got)
+    acc, yg = torch.ones_like(got), to_gpu(y)
+    _lib.check(_lib.load().cbct_fdk(geom.handle, yg.data_ptr(), acc.data_ptr(), 2, 1,
+                                    torch.cuda.current_stream().cuda_stream))
+    assert float((acc - 1.0 - got).abs().max()) <= 1e-6 * (1.0 + float(got.abs().max()))
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), 3e38])
+@pytest.mark.parametrize("name", ["fft1024", "direct_small_split"])
+def test_non_finite_row_stays_in_its_row(O, name, value):
+    g = CASES[name]
+    geom = P.Geometry(g)
+    y = to_gpu(I.random_volume((1,) + geom.proj_shape, 6))
+    clean = ops.fdk(geom, y)
+    k, iv = 5, 12
+    y[0, k, iv, 40:44] = value
+    got = ops.fdk(geom, y)
+    # detector row of every voxel at that angle
+    z, yy, x = (torch.arange(n, device="cuda", dtype=torch.float64) - 0.5 * (n - 1) for n in geom.vol_shape)
+    th = 2 * np.pi * k / g["n_angles"]
+    U = 1000.0 - 4.0 * (x[None, :] * np.cos(th) + yy[:, None] * np.sin(th))
+    fv = (1536.0 / U)[None] * (4.0 * z)[:, None, None] / g["dv"] + 0.5 * (g["nv"] - 1)
+    far = ((fv - iv).abs() > 1.01)[None]
+    assert float((got[far] - clean[far]).abs().max()) <= 1e-6 * float(clean.abs().max())
+    near = ((fv - iv).abs() < 0.9)[None]
+    assert int(near.sum()) > 100
+    if value != 3e38:
+        assert int((~torch.isfinite(got[near])).sum()) > 50
