@@ -249,6 +249,17 @@ __device__ __forceinline__ void tile_next(TileCoord &c, int D, int nh, int W) {
     ++c.img;
 }
 
+// Advances c by a step of fewer tiles than there are in the image stack, given as a TileCoord.
+__device__ __forceinline__ void tile_step(TileCoord &c, const TileCoord &st, int D, int nh, int ntw) {
+    c.w0 += st.w0;
+    c.th += st.th;
+    c.d += st.d;
+    c.img += st.img;
+    if (c.w0 >= 128 * ntw) { c.w0 -= 128 * ntw; ++c.th; }
+    if (c.th >= nh) { c.th -= nh; ++c.d; }
+    if (c.d >= D) { c.d -= D; ++c.img; }
+}
+
 // Warp-specialized convolution over row-halo stages. Item i of a CTA = (tile
 // t_begin + i / nch, input plane dd = i % nch - 1 for 3-D, the tile's own plane for
 // 2-D) on ring stage i % nst.
@@ -574,10 +585,13 @@ __global__ void k_pack_jobs(const ConvPackJob *__restrict__ jobs, const float *_
 // K stride 128 B) and B = both dY rows (N = 2 x 8 NCG: core matrix (o, g) at (o NCG + g)
 // 2048 B) accumulates D_dw[(r, ci)][(o, co)] in TMEM over every tile of the CTA. Entry
 // (r, o) belongs to tap dh = r - 1 - o: six of the eight (r, o) pairs are taps, and two
-// pairs give each tap, so each CTA writes both (o = 0, 1) partials of its 9 taps and a
-// fixed-order reduction adds everything (deterministic). Two dY rows per MMA halve the
-// MMA count per output row, and the three taps dd in separate CTAs keep the accumulators
-// at 3 x N <= 192 TMEM columns, so two CTAs (two MMA issuers) share an SM.
+// pairs (o = 0, 1) give each tap: the epilogue adds them through shared memory, each CTA writes
+// one partial of its 9 taps and a fixed-order reduction adds the CTAs (deterministic). Two dY rows
+// per MMA halve the MMA count per output row, and the three taps dd in separate CTAs keep the
+// accumulators at 3 x N <= 192 TMEM columns, so two CTAs (two MMA issuers) share an SM.
+// The bias gradient is summed by the epilogue warps of the middle depth tap's CTAs from the dY
+// rows in the stages, while the MMAs run (a pass of its own over dY took 35 us, its one-CTA reduction
+// 52 us at 128^3 x 32 channels).
 constexpr int kWgThreads = 192;  // warps 0-3 epilogue, 4 TMA producer, 5 MMA
 constexpr int kWgStages = 2;
 constexpr int kWgXBytes = 4 * 4 * kRowStride;  // 4 input rows x 4 channel groups
@@ -589,11 +603,16 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32_mn(int M, int N) {
 // XCG = input channel groups (4, or 1 for 8-channel inputs: each input row is then
 // loaded to region 4 r and the regions of groups 1..3 stay zero); NCG = output-channel
 // groups per dY row: 2 (16 outputs, the second group zero when cout <= 8) or 4.
-// partial: [ndd][gridDim.x][2][cout][9][cin].
+// Grid: ndd x gpd CTAs, the depth taps of a range of tiles next to each other: they run at the
+// same time on the same planes, and the tiles of a CTA are gpd apart, so that all CTAs move through the
+// planes together and read them from L2 (at 128^3 x 32 channels: 268 MB and 127 us, the MMAs now the limit; with the taps as three successive
+// waves every plane came from DRAM three times, 813 MB, 78 % of the DRAM rate).
+// partial: [ndd][gpd][cout][9][cin]; partial_b (null without a bias): [gpd][cout].
 template <int XCG, int NCG>
 __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_constant__ CUtensorMap xmap,
                                                               const __grid_constant__ CUtensorMap ymap, ConvArgs a,
-                                                              int cgo, float *__restrict__ partial) {
+                                                              int cgo, float *__restrict__ partial,
+                                                              float *__restrict__ partial_b) {
     constexpr int kN = 2 * NCG * 8;
     constexpr int kYBytes = 2 * NCG * 2048;
     constexpr int kStage = kWgXBytes + kYBytes;
@@ -607,7 +626,10 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
     int *abort_flag = reinterpret_cast<int *>(tmem_slot + 1);
     int *used = abort_flag + 1;  // [3]: accumulator dw received an MMA
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int dd = blockIdx.y;   // depth tap (3-D: input plane d + dd - 1)
+    const int ndd = a.taps3d ? 3 : 1, gpd = (int)gridDim.x / ndd;
+    const int dd = blockIdx.x % ndd, cta = blockIdx.x / ndd;  // depth tap (3-D: input plane d + dd - 1), its CTA
+    const bool bias = partial_b && dd == (a.taps3d ? 1 : 0);  // (the middle tap's input plane always exists)
+    static_assert(9 * 32 * 32 * sizeof(float) <= kWgStages * (kWgXBytes + 2 * 2 * 2048), "tap sums in the stages");
     constexpr uint32_t kIdesc = idesc_bf16_f32_mn(128, kN);
     const int rs = 16 * a.G * conv_box_rows(a.G);
 
@@ -615,7 +637,7 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
     if (tid == 32) {
         for (int s = 0; s < kWgStages; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
+            mbar_init(&empty[s], bias ? 5 : 1);  // the MMAs' commit (and the four epilogue warps)
         }
         mbar_init(done, 2);  // the MMAs' commit + the MMA thread's release of used[]
         *abort_flag = 0;
@@ -648,9 +670,9 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
 
     const int ntw = (a.W + 127) / 128, nh = (a.H + 1) / 2;
     const long long ntiles = (long long)a.nimg * a.D * nh * ntw;
-    const long long per_cta = (ntiles + gridDim.x - 1) / gridDim.x;
-    const long long t_begin = (long long)blockIdx.x * per_cta;
-    const long long my_tiles = t_begin < ntiles ? min(per_cta, ntiles - t_begin) : 0;
+    // tiles cta, cta + gpd, ...: the CTAs move through the planes together
+    const long long t_begin = cta, my_tiles = cta < ntiles ? (ntiles - cta + gpd - 1) / gpd : 0;
+    const TileCoord step = tile_coord(gpd, a.D, nh, ntw);
     const uint32_t sm_u = smem_u32(sm);
 
     if (warp == 4) {
@@ -685,7 +707,7 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
                         tma_load_5d(st + (uint32_t)(kWgXBytes + o * NCG * 2048), &ymap, 0, tc.w0 / a.G, 0,
                                     2 * tc.th + o, tc.img * a.D + tc.d, &full[s]);
                 }
-                tile_next(tc, a.D, nh, a.W);
+                tile_step(tc, step, a.D, nh, ntw);
                 if (++s == kWgStages) {
                     s = 0;
                     ph ^= 1u;
@@ -722,7 +744,7 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
                     }
                 }
                 mma_commit(&empty[s]);
-                tile_next(tc, a.D, nh, a.W);
+                tile_step(tc, step, a.D, nh, ntw);
                 if (++s == kWgStages) {
                     s = 0;
                     ph ^= 1u;
@@ -736,28 +758,83 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
             mbar_arrive(done);
         }
     } else {
-        // epilogue (warps 0-3, once): warp w holds accumulator rows 32 w .. 32 w + 31 = input
-        // row r = w, input channel = lane; columns (o, co). Pair (r, o) is tap dh = r - 1 - o.
+        if (bias) {
+            // warp = output-channel group, lane = pixels lane, lane + 32, ... of both dY rows (zero
+            // outside the image)
+            float sum[8] = {};
+            int s = 0;
+            uint32_t ph = 0;
+            for (long long i = 0; i < my_tiles; ++i) {
+                if (!mbar_wait(&full[s], ph, a.status)) {
+                    *abort_flag = 1;
+                    break;
+                }
+                if (warp < cgo) {
+                    const uint4 *src = reinterpret_cast<const uint4 *>(sm + s * kStage + kWgXBytes + warp * 2048) + lane;
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const uint4 v = src[(e >> 2) * NCG * 128 + (e & 3) * 32];
+                        const __nv_bfloat162 *p = reinterpret_cast<const __nv_bfloat162 *>(&v);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const float2 f = __bfloat1622float2(p[j]);
+                            sum[2 * j] += f.x;
+                            sum[2 * j + 1] += f.y;
+                        }
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&empty[s]);
+                if (++s == kWgStages) {
+                    s = 0;
+                    ph ^= 1u;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) sum[j] += __shfl_xor_sync(0xffffffffu, sum[j], o);
+                const int co = 8 * warp + j;
+                if (lane == 0 && warp < cgo && co < a.cout) partial_b[(long long)cta * a.cout + co] = sum[j];
+            }
+        }
+        // epilogue (warps 0-3): warp w holds accumulator rows 32 w .. 32 w + 31 = input
+        // row r = w, input channel = lane; columns (o, co). Pair (r, o) is tap dh = r - 1 - o: row r's
+        // o = 1 columns go through shared memory (the stages are free) to row r - 1's o = 0 ones
         const bool ok = mbar_wait(done, 0u, a.status);
         tc_fence_after();
-        const int r = warp, ci = lane;
-        const long long slot = ((long long)dd * gridDim.x + blockIdx.x) * 2;
+        float *tap = reinterpret_cast<float *>(sm);  // [dw][dh + 1][co][32]
+        constexpr int kTap = NCG * 8 * 32;
         const long long per_o = (long long)a.cout * 9 * a.cin;
-        for (int dw = 0; dw < 3; ++dw) {
-            float v[kN];
+        float *pb = partial + ((long long)dd * gpd + cta) * per_o;
+        if (warp >= 1) {
+#pragma unroll 1
+            for (int dw = 0; dw < 3; ++dw)
 #pragma unroll
-            for (int c0 = 0; c0 < kN; c0 += 16)
-                tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(dw * kN + c0), v + c0);
-            const bool valid = ok && !*abort_flag && used[dw];
+                for (int c0 = 0; c0 < NCG * 8; c0 += 16) {
+                    float v[16];
+                    tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(dw * kN + NCG * 8 + c0), v);
 #pragma unroll
-            for (int o = 0; o < 2; ++o) {
-                const int dh = r - 1 - o;
-                if (dh < -1 || dh > 1 || ci >= a.cin) continue;
-                float *pb = partial + (slot + o) * per_o;
-                const int t9 = (dh + 1) * 3 + dw;
+                    for (int j = 0; j < 16; ++j) tap[(dw * 3 + warp - 1) * kTap + (c0 + j) * 32 + lane] = v[j];
+                }
+        }
+        asm volatile("bar.sync 1, 128;" ::: "memory");  // the four epilogue warps
+        if (warp < 3) {
+#pragma unroll 1
+            for (int dw = 0; dw < 3; ++dw) {
+                const bool valid = ok && !*abort_flag && used[dw];
 #pragma unroll
-                for (int co = 0; co < NCG * 8; ++co)
-                    if (co < a.cout) pb[((long long)co * 9 + t9) * a.cin + ci] = valid ? v[o * NCG * 8 + co] : 0.f;
+                for (int c0 = 0; c0 < NCG * 8; c0 += 16) {
+                    float v[16];
+                    tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(dw * kN + c0), v);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        const int co = c0 + j;
+                        if (lane < a.cin && co < a.cout)
+                            pb[((long long)co * 9 + warp * 3 + dw) * a.cin + lane] =
+                                valid ? v[j] + tap[(dw * 3 + warp) * kTap + co * 32 + lane] : 0.f;
+                    }
+                }
             }
         }
     }
@@ -769,55 +846,36 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
     }
 }
 
-// out[co0 + co][tap][ci0 + ci] (+)= sum over the CTAs of their tap's partials (both
-// output-row halves), fixed order: partial [ndd][gpd][2][cout][9][cin], tap = dd * 9 + t9;
-// out has cin_full input channels per tap.
-__global__ void k_reduce_wgrad(const float *__restrict__ partial, int gpd, int ndd, int cout, int cin,
-                               float *__restrict__ out, int accumulate, int co0, int ci0, int cin_full) {
-    const int n = cout * 9 * ndd * cin;
-    const long long per_o = (long long)cout * 9 * cin;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int ci = i % cin, tap = (i / cin) % (9 * ndd), co = i / (cin * 9 * ndd);
-        const int d = tap / 9, t9 = tap % 9;
-        const long long e = ((long long)co * 9 + t9) * cin + ci;
-        const long long o = ((long long)(co0 + co) * 9 * ndd + tap) * cin_full + ci0 + ci;
-        float s = accumulate ? out[o] : 0.f;
-        for (int b = 0; b < gpd; ++b) {
-            const float *p = partial + ((long long)d * gpd + b) * 2 * per_o;
-            s += p[e] + p[per_o + e];
-        }
-        out[o] = s;
+// out[co0 + co][tap][ci0 + ci] (+)= sum over the CTAs of their tap's partials, fixed order: partial
+// [ndd][gpd][cout][9][cin], tap = dd * 9 + t9; out has cin_full input channels per tap. The
+// blocks past the weights' sum the bias partials partial_b [gpd][cout] into db. A block takes 32
+// sums, each as 8 slices of the CTAs added in order: enough loads in flight to read the partials at L2
+// speed (one thread per sum took 65 us for 67 MB; now 10 us for 34 MB).
+__global__ void __launch_bounds__(256) k_reduce_wgrad(const float *__restrict__ partial, int gpd, int ndd, int cout, int cin,
+                                                      float *__restrict__ out, int accumulate, int co0, int ci0, int cin_full,
+                                                      const float *__restrict__ partial_b, float *__restrict__ db) {
+    __shared__ float red[8][32];
+    const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
+    const int n = cout * 9 * ndd * cin, wblocks = (n + 31) / 32;
+    const bool is_b = (int)blockIdx.x >= wblocks;
+    const int i = (is_b ? (int)blockIdx.x - wblocks : (int)blockIdx.x) * 32 + lane;
+    const bool ok = i < (is_b ? cout : n);
+    const int ci = i % cin, tap = (i / cin) % (9 * ndd), co = i / (cin * 9 * ndd), d = tap / 9, t9 = tap % 9;
+    const long long stride = is_b ? cout : (long long)cout * 9 * cin;
+    const float *p = is_b ? partial_b + i : partial + (long long)d * gpd * stride + ((long long)co * 9 + t9) * cin + ci;
+    float s = 0.f;
+    if (ok) {
+        const int b1 = gpd * (sl + 1) / 8;
+#pragma unroll 8
+        for (int b = gpd * sl / 8; b < b1; ++b) s += p[b * stride];
     }
-}
-
-// partial_b[blk][co] = sum over the block's image rows of dY[row][co] (row-blocked dY,
-// cgo channel groups read, rows cgs groups apart): thread (group q, column lane) reads
-// 16-byte pixels along the row, then the lanes of each channel are summed in a fixed order.
-__global__ void __launch_bounds__(256) k_bias_grad(const __nv_bfloat16 *__restrict__ dy, int cgo, int cgs, int cout,
-                                                   long long nrows, int W, int rows_per_block,
-                                                   float *__restrict__ partial_b) {
-    __shared__ float red[256][9];
-    const int tpq = 256 / cgo, q = threadIdx.x / tpq, l = threadIdx.x - q * tpq;
-    const long long r0 = (long long)blockIdx.x * rows_per_block, r1 = min(nrows, r0 + rows_per_block);
-    float acc[8] = {};
-    for (long long row = r0; row < r1; ++row) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(dy + (row * cgs + q) * (long long)W * 8);
-        for (int w = l; w < W; w += tpq) {
-            const uint4 v = __ldg(src + w);
-            const __nv_bfloat16 *b = reinterpret_cast<const __nv_bfloat16 *>(&v);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) acc[j] += __bfloat162float(b[j]);
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) red[threadIdx.x][j] = acc[j];
+    red[sl][lane] = s;
     __syncthreads();
-    const int c = threadIdx.x;
-    if (c < cout) {
-        const int qc = c / 8, j = c % 8;
-        float t = 0.f;
-        for (int k = 0; k < tpq; ++k) t += red[qc * tpq + k][j];
-        partial_b[(long long)blockIdx.x * cout + c] = t;
+    if (sl == 0 && ok) {
+        float *o = is_b ? db + co0 + i : out + ((long long)(co0 + co) * 9 * ndd + tap) * cin_full + ci0 + ci;
+        float t = accumulate ? *o : 0.f;
+        for (int k = 0; k < 8; ++k) t += red[k][lane];
+        *o = t;
     }
 }
 
@@ -1029,7 +1087,7 @@ static int conv_run(const ConvArgs &a0, int n_out, int epi, int rpt, cudaStream_
 // input slots of rows xgs channel groups apart (a view into a wider input), dy cgo output
 // groups of rows ygs groups apart. dw[co0 + co][tap][ci0 + ci] (cin_full channels per tap)
 // (+)= the block's per-CTA partials, reduced in a fixed order; db[co0 + co] (+)= the bias
-// gradient when db is not null (CUDA cores).
+// gradient when db is not null.
 template <int XCG, int NCG>
 static int conv_wgrad_tc(const __nv_bfloat16 *x, int xgs, int cin, const __nv_bfloat16 *dy, int cgo, int ygs,
                          int cout, int nimg, int D, int H, int W, int taps3d, float *dw, int co0, int ci0,
@@ -1064,22 +1122,15 @@ static int conv_wgrad_tc(const __nv_bfloat16 *x, int xgs, int cin, const __nv_bf
     const int nsm = sm_count();
     const int ndd = taps3d ? 3 : 1;
     const long long ntiles = (long long)nimg * D * ((H + 1) / 2) * ((W + 127) / 128);
-    const int gpd = (int)std::max<long long>(1, std::min<long long>(ntiles, 2LL * nsm));  // CTAs per depth tap
-    const long long per_cta = 2LL * cout * 9 * cin;
+    const int gpd = (int)std::max<long long>(1, std::min<long long>(ntiles, 2LL * nsm / ndd));  // CTAs per depth tap
+    const long long per_cta = (long long)cout * 9 * cin;
     const int nw = cout * 9 * ndd * cin;
-    const long long nrows = (long long)nimg * D * H;
-    const int nbb = (int)std::min<long long>(4LL * nsm, nrows);
-    const int rpb = (int)((nrows + nbb - 1) / nbb);
     float *part = nullptr;
-    CBCT_CUDA_TRY(cudaMallocAsync((void **)&part, sizeof(float) * ((long long)ndd * gpd * per_cta + (long long)nbb * cout),
-                                  st));
-    float *partb = part + (long long)ndd * gpd * per_cta;
-    k_conv_wgrad_tc<XCG, NCG><<<dim3(gpd, ndd), kWgThreads, smem, st>>>(xmap, ymap, a, cgo, part);
-    k_reduce_wgrad<<<(nw + 255) / 256, 256, 0, st>>>(part, gpd, ndd, cout, cin, dw, accumulate, co0, ci0, cin_full);
-    if (db) {
-        k_bias_grad<<<nbb, 256, 0, st>>>(dy, cgo, ygs, cout, nrows, W, rpb, partb);
-        k_reduce_rows<<<1, 256, 0, st>>>(partb, nbb, cout, db + co0, accumulate);
-    }
+    CBCT_CUDA_TRY(cudaMallocAsync((void **)&part, sizeof(float) * ((long long)ndd * gpd * per_cta + (long long)gpd * cout), st));
+    float *partb = db ? part + (long long)ndd * gpd * per_cta : nullptr;
+    k_conv_wgrad_tc<XCG, NCG><<<gpd * ndd, kWgThreads, smem, st>>>(xmap, ymap, a, cgo, part, partb);
+    k_reduce_wgrad<<<(nw + 31) / 32 + (db ? (cout + 31) / 32 : 0), 256, 0, st>>>(part, gpd, ndd, cout, cin, dw, accumulate, co0,
+                                                                               ci0, cin_full, partb, db);
     cudaError_t e = cudaGetLastError();
     cudaFreeAsync(part, st);
     if (e != cudaSuccess) return cuda_fail(e, "conv wgrad (tensor cores)");
