@@ -20,8 +20,9 @@
  *        volume      [batch][nz][ny][nx]       (x fastest)
  *        projection  [batch][n_angles][nv][nu] (u fastest)
  *  - The library owns geometry tables, weights and workspaces behind opaque
- *    handles. Scratch memory is taken from the CUDA stream-ordered pool on the
- *    caller's stream (cudaMallocAsync) and returned on the same stream.
+ *    handles. Scratch memory is taken from a stream-ordered pool of the library on
+ *    the caller's stream and returned on the same stream; while a geometry exists on
+ *    a device, up to 1 GiB of it stays reserved between calls.
  *  - Calls are asynchronous on `stream` (a cudaStream_t; 0 = legacy default) and
  *    never synchronise the device.
  *  - Return value: 0 on success, negative on error; cbct_last_error() returns a

@@ -107,6 +107,8 @@ class CbctError(RuntimeError):
 def load():
     """Load libcbct.so (raises if it is absent: there is no CPU fallback)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):

@@ -161,6 +161,14 @@ __device__ __forceinline__ long long vox_index(const GeomDev &g, int ix, int iy,
 // of the grid-size heuristics.
 int sm_count();
 
+// Stream-ordered scratch memory of the current device for a call on `st` (returned with
+// cudaFreeAsync). While a geometry exists on the device, up to kScratchKept bytes stay with the
+// library between calls instead of going back to the driver at every synchronisation.
+constexpr size_t kScratchKept = 1ull << 30;
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t st);
+void scratch_retain(int dev);   // a geometry was made on dev
+void scratch_release(int dev);  // and destroyed (with the device idle): the last one gives the memory back
+
 // Host-side geometry object.
 struct Geom;
 GeomDev dev_view(const cbct_geom *g);

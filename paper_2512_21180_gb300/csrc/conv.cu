@@ -1126,7 +1126,7 @@ static int conv_wgrad_tc(const __nv_bfloat16 *x, int xgs, int cin, const __nv_bf
     const long long per_cta = (long long)cout * 9 * cin;
     const int nw = cout * 9 * ndd * cin;
     float *part = nullptr;
-    CBCT_CUDA_TRY(cudaMallocAsync((void **)&part, sizeof(float) * ((long long)ndd * gpd * per_cta + (long long)gpd * cout), st));
+    CBCT_CUDA_TRY(scratch_alloc((void **)&part, sizeof(float) * ((long long)ndd * gpd * per_cta + (long long)gpd * cout), st));
     float *partb = db ? part + (long long)ndd * gpd * per_cta : nullptr;
     k_conv_wgrad_tc<XCG, NCG><<<gpd * ndd, kWgThreads, smem, st>>>(xmap, ymap, a, cgo, part, partb);
     k_reduce_wgrad<<<(nw + 31) / 32 + (db ? (cout + 31) / 32 : 0), 256, 0, st>>>(part, gpd, ndd, cout, cin, dw, accumulate, co0,
@@ -1175,7 +1175,7 @@ int conv_wgrad(const __nv_bfloat16 *x, int cpin, int cin, const __nv_bfloat16 *d
     const int ppb = (int)((npix + nblk - 1) / nblk);
     const int nw = cout * ntaps * cin;
     float *part = nullptr;
-    CBCT_CUDA_TRY(cudaMallocAsync((void **)&part, sizeof(float) * (long long)nblk * (nw + cout), st));
+    CBCT_CUDA_TRY(scratch_alloc((void **)&part, sizeof(float) * (long long)nblk * (nw + cout), st));
     float *partb = part + (long long)nblk * nw;
     k_conv_wgrad<<<nblk, 256, 0, st>>>(x, cpin, cin, dy, cpout, cout, nimg, D, H, W, taps3d, ppb, part, partb);
     k_reduce_rows<<<(nw + 255) / 256, 256, 0, st>>>(part, nblk, nw, dw, accumulate);
@@ -1247,7 +1247,7 @@ int cbct::conv_apply(const void *x, int nimg, int D, int H, int W, int cpin, int
     uint8_t *pk = nullptr;
     int rc = 0;
     if (!packed) {
-        CBCT_CUDA_TRY(cudaMallocAsync((void **)&pk, bytes, st));
+        CBCT_CUDA_TRY(scratch_alloc((void **)&pk, bytes, st));
         for (int h = 0; h < conv_halves(n_out) && rc == 0; ++h)
             rc = conv_pack(w, cout, taps3d, cin, cpin, flip, jobs[h].rpt, jobs[h].o0, conv_half_nout(n_out, h),
                            pk + jobs[h].out_off, st);

@@ -20,6 +20,7 @@ struct cbct_geom {
     float2 *cs32 = nullptr;                // [na] (cos, sin) of each angle, for FDK
     cbct::GeomDev dev{};                   // kernel view
     int *status = nullptr;                 // device status word of this geometry's kernels
+    bool scratch = false;                  // counted by scratch_retain
     int fwd_cfg = -1;                      // staged forward box configuration, -1: direct kernel
     double fwd_need_b = 0.0, fwd_need_z = 0.0;  // host bounds of a tile's chunk footprint
     bool axis_contiguous = true;           // x- and y-principal columns form intervals at every angle

@@ -9,9 +9,11 @@
 // with a = -(nu-1)/2 du + u_offset and b = -(nv-1)/2 dv + v_offset, evaluated in
 // FP64 on the host in this order and rounded once to FP32 for the kernels.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -48,6 +50,66 @@ int sm_count() {
         cached[dev] = n;
     }
     return cached[dev];
+}
+
+// One memory pool per device. The default pool returns its memory to the driver whenever the device
+// synchronises, so that a program that waits for each result paid for new mappings on every call:
+// 16^3 forward and adjoint 250 us instead of 40, one clinical FDK 2.3 ms more (CUDA 13.0). The
+// library's own pool keeps up to kScratchKept bytes while a geometry exists and nothing afterwards; the
+// driver orders its reuse across streams and threads.
+namespace {
+constexpr int kMaxPools = 64;
+std::mutex g_pool_mu;
+std::atomic<cudaMemPool_t> g_pool[kMaxPools];
+int g_pool_refs[kMaxPools];
+
+cudaMemPool_t pool_of(int dev) {
+    if (dev < 0 || dev >= kMaxPools) return nullptr;
+    cudaMemPool_t p = g_pool[dev].load(std::memory_order_acquire);
+    if (p) return p;
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    p = g_pool[dev].load(std::memory_order_relaxed);
+    if (!p) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        if (cudaMemPoolCreate(&p, &props) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        g_pool[dev].store(p, std::memory_order_release);
+    }
+    return p;
+}
+
+void pool_keep(cudaMemPool_t p, unsigned long long bytes) {
+    if (p) cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &bytes);
+}
+}  // namespace
+
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t st) {
+    int dev = -1;
+    cudaGetDevice(&dev);
+    const cudaMemPool_t pool = pool_of(dev);
+    return pool ? cudaMallocFromPoolAsync(p, bytes, pool, st) : cudaMallocAsync(p, bytes, st);
+}
+
+void scratch_retain(int dev) {
+    const cudaMemPool_t p = pool_of(dev);
+    if (!p) return;
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    if (g_pool_refs[dev]++ == 0) pool_keep(p, kScratchKept);
+}
+
+void scratch_release(int dev) {
+    const cudaMemPool_t p = pool_of(dev);
+    if (!p) return;
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    if (--g_pool_refs[dev] == 0) {
+        pool_keep(p, 0);
+        cudaMemPoolTrimTo(p, 0);
+    }
 }
 
 }  // namespace cbct
@@ -289,6 +351,8 @@ extern "C" int geometry_create(const cbct_geom_desc *desc, cbct_geom **out) {
         v.scaled = 1.0 / nrm;
         v.scale = (float)v.scaled;
     }
+    cbct::scratch_retain(dev);
+    g->scratch = true;
     *out = g;
     return 0;
 }
@@ -307,6 +371,7 @@ extern "C" void geometry_destroy(cbct_geom *g) {
     if (g->rz64) cudaFree(g->rz64);
     if (g->cs32) cudaFree(g->cs32);
     if (g->status) cudaFree(g->status);
+    if (g->scratch) cbct::scratch_release(g->device);
     cudaSetDevice(cur);
     delete g;
 }

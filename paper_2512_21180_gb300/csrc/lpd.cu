@@ -1873,7 +1873,7 @@ extern "C" int cbct_masked_mse(const float *x, const float *ref, const float *V,
     cudaStream_t st = (cudaStream_t)stream;
     const int nb = 256;
     double *part = nullptr;
-    CBCT_CUDA_TRY(cudaMallocAsync((void **)&part, sizeof(double) * 2 * nb + 16, st));
+    CBCT_CUDA_TRY(scratch_alloc((void **)&part, sizeof(double) * 2 * nb + 16, st));
     float *cnt = reinterpret_cast<float *>(part + 2 * nb);
     k_mse_partial<<<nb, 256, 0, st>>>(x, ref, V, thr, n, part, part + nb);
     k_mse_final<<<1, 1, 0, st>>>(part, part + nb, nb, loss, cnt);

@@ -669,7 +669,7 @@ static int backward_impl(const cbct_geom *g, const T *proj, T *vol, int batch, i
     // the segment gather loads the weighted projections by TMA: rows start on 16 bytes
     const int pitch = sizeof(T) == 4 && g->axis_contiguous ? (d.nu + 3) & ~3 : d.nu;
     T *pw = nullptr;
-    CBCT_CUDA_TRY(cudaMallocAsync((void **)&pw, sizeof(T) * (nproj / d.nu) * pitch, st));
+    CBCT_CUDA_TRY(scratch_alloc((void **)&pw, sizeof(T) * (nproj / d.nu) * pitch, st));
     dim3 blk(32, 8), gw((d.nu + 31) / 32, (d.nv + 7) / 8, d.na * batch);
     k_weight_rays<T><<<gw, blk, 0, st>>>(d, proj, pw, colw, pitch);
     cudaError_t e = cudaGetLastError();
@@ -689,7 +689,7 @@ static int backward_impl(const cbct_geom *g, const T *proj, T *vol, int batch, i
                 if ((long long)nzb * batch * nparts > 65535) e = cudaErrorInvalidConfiguration;
                 float *partial = nullptr;
                 const long long nvol = (long long)batch * d.n[0] * d.n[1] * d.n[2];
-                if (e == cudaSuccess && nparts > 1) e = cudaMallocAsync((void **)&partial, sizeof(float) * nvol * nparts, st);
+                if (e == cudaSuccess && nparts > 1) e = scratch_alloc((void **)&partial, sizeof(float) * nvol * nparts, st);
                 int trc = 0;
                 if (e == cudaSuccess) {
                     CUtensorMap pmap;
@@ -796,7 +796,7 @@ extern "C" int cbct_count_samples(const cbct_geom *g, long long *out, void *stre
     if (!g || !out) return fail(CBCT_EINVAL, "cbct_count_samples: NULL argument");
     cudaStream_t st = (cudaStream_t)stream;
     unsigned long long *d = nullptr, h = 0;
-    CBCT_CUDA_TRY(cudaMallocAsync((void **)&d, sizeof(unsigned long long), st));
+    CBCT_CUDA_TRY(scratch_alloc((void **)&d, sizeof(unsigned long long), st));
     cudaMemsetAsync(d, 0, sizeof(unsigned long long), st);
     const GeomDev &v = g->dev;
     dim3 blk(32, 8), grd((v.nu + 31) / 32, (v.nv + 7) / 8, v.na);

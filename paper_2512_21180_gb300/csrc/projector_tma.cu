@@ -455,7 +455,7 @@ int forward_staged(const cbct_geom *g, const float *vol, float *proj, int batch,
     const int px = (ny + 3) & ~3, py = (nx + 3) & ~3;
     const long long ex = (long long)batch * nx * nz * px, ey = copy_y ? (long long)batch * ny * nz * py : 0;
     float *buf = nullptr;
-    CBCT_CUDA_TRY(cudaMallocAsync((void **)&buf, sizeof(float) * (ex + ey), st));
+    CBCT_CUDA_TRY(scratch_alloc((void **)&buf, sizeof(float) * (ex + ey), st));
     float *tx = buf, *ty = buf + ex;
     const PlaneView vx{tx, (long long)nx * nz * px, (long long)nz * px, px};
     const PlaneView vy = copy_y ? PlaneView{ty, (long long)ny * nz * py, (long long)nz * py, py}

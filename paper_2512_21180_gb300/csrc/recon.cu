@@ -571,7 +571,7 @@ extern "C" int cbct_fdk(const cbct_geom *g, const float *proj, float *vol, int b
     // the direct filter
     const long long nq0 = nfft ? 0 : padded(rows * nue), nq = padded((long long)batch * d.n_angles * (d.nv + 2) * (nue + 2));
     float *q0 = nullptr, *q = nullptr, *w = nullptr;
-    CBCT_CUDA_TRY(cudaMallocAsync((void **)&q0, sizeof(float) * (nq0 + nq + padded(d.nu) + nfft + npart), st));
+    CBCT_CUDA_TRY(scratch_alloc((void **)&q0, sizeof(float) * (nq0 + nq + padded(d.nu) + nfft + npart), st));
     q = q0 + nq0;
     w = q + nq;
     float *H = w + padded(d.nu), *partial = H + nfft;
@@ -617,7 +617,7 @@ extern "C" int cbct_opnorm(const cbct_geom *g, double gamma, int iters, double *
     const long long nvox = (long long)d.n[0] * d.n[1] * d.n[2], nproj = (long long)d.na * d.nv * d.nu;
     float *x = nullptr, *p = nullptr, *y = nullptr;
     double *acc = nullptr;
-    CBCT_CUDA_TRY(cudaMallocAsync((void **)&x, sizeof(float) * (2 * padded(nvox) + padded(nproj)) + 16, st));
+    CBCT_CUDA_TRY(scratch_alloc((void **)&x, sizeof(float) * (2 * padded(nvox) + padded(nproj)) + 16, st));
     y = x + padded(nvox);
     p = y + padded(nvox);
     acc = reinterpret_cast<double *>(p + padded(nproj));
@@ -658,7 +658,7 @@ extern "C" int cbct_pdhg(const cbct_geom *g, const float *y, const float *x0, fl
     float *buf = nullptr;
     // xbar, bt (N each), z2 (3N), z1, p (M each)
     const long long Np = padded(N), Mp = padded(M), N3 = padded(3 * N);
-    CBCT_CUDA_TRY(cudaMallocAsync((void **)&buf, sizeof(float) * (2 * Np + N3 + 2 * Mp), st));
+    CBCT_CUDA_TRY(scratch_alloc((void **)&buf, sizeof(float) * (2 * Np + N3 + 2 * Mp), st));
     float *xb = buf, *bt = xb + Np, *z2 = bt + Np, *z1 = z2 + N3, *p = z1 + Mp;
     if (x != x0) cudaMemcpyAsync(x, x0, sizeof(float) * N, cudaMemcpyDeviceToDevice, st);
     cudaMemcpyAsync(xb, x0, sizeof(float) * N, cudaMemcpyDeviceToDevice, st);
@@ -689,7 +689,7 @@ extern "C" int cbct_landweber(const cbct_geom *g, const float *y, float *x, int 
     const GeomDev &d = g->dev;
     const long long N = (long long)batch * d.n[0] * d.n[1] * d.n[2], M = (long long)batch * d.na * d.nv * d.nu;
     float *buf = nullptr;
-    CBCT_CUDA_TRY(cudaMallocAsync((void **)&buf, sizeof(float) * (padded(N) + M), st));
+    CBCT_CUDA_TRY(scratch_alloc((void **)&buf, sizeof(float) * (padded(N) + M), st));
     float *gr = buf, *r = buf + padded(N);
     int rc = 0;
     for (int it = 0; it < niter && rc == 0; ++it) {

@@ -306,7 +306,7 @@ extern "C" int cbct_phantom(const cbct_geom *g, const double *ell_host, int n_el
     cudaStream_t st = (cudaStream_t)stream;
     double *d = nullptr;
     if (n_ell > 0) {
-        CBCT_CUDA_TRY(cudaMallocAsync((void **)&d, sizeof(double) * 17 * n_ell, st));
+        CBCT_CUDA_TRY(scratch_alloc((void **)&d, sizeof(double) * 17 * n_ell, st));
         cudaError_t e = cudaMemcpyAsync(d, ell_host, sizeof(double) * 17 * n_ell, cudaMemcpyHostToDevice, st);
         if (e != cudaSuccess) { cudaFreeAsync(d, st); return cuda_fail(e, "cbct_phantom: upload"); }
     }
@@ -372,7 +372,7 @@ extern "C" int cbct_fov(const cbct_geom *g, float *V, void *stream) {
         cs[2 * k + 1] = sin(th);
     }
     double *dcs = nullptr;
-    CBCT_CUDA_TRY(cudaMallocAsync((void **)&dcs, sizeof(double) * cs.size(), st));
+    CBCT_CUDA_TRY(scratch_alloc((void **)&dcs, sizeof(double) * cs.size(), st));
     cudaError_t e = cudaMemcpyAsync(dcs, cs.data(), sizeof(double) * cs.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) {
         const long long nvox = (long long)d.nx * d.ny * d.nz;
@@ -433,7 +433,7 @@ extern "C" int cbct_poly_simulate(const cbct_geom *g, const float *mu, int batch
     const long long nvox = (long long)v.n[0] * v.n[1] * v.n[2];
     const long long per_item = (long long)v.na * v.nv * v.nu;
     float *rho = nullptr;
-    CBCT_CUDA_TRY(cudaMallocAsync((void **)&rho, sizeof(float) * 2 * nvox * batch, st));
+    CBCT_CUDA_TRY(scratch_alloc((void **)&rho, sizeof(float) * 2 * nvox * batch, st));
     k_water_bone<<<grid_for(nvox * batch), 256, 0, st>>>(mu, nvox, nvox * batch, (float)mu_water60, rho);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {

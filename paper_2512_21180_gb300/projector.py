@@ -102,6 +102,18 @@ def _batched(t: torch.Tensor, shape, what: str):
     return t.contiguous()
 
 
+def _run(fn, what: str, t: torch.Tensor, *args):
+    """fn(*args, stream) on t's device and its current stream (the device guard only when another
+    device is current: it costs as much as a small kernel's launch)."""
+    if torch.cuda.current_device() == t.device.index:
+        rc = fn(*args, _stream(t))
+    else:
+        with torch.cuda.device(t.device):
+            rc = fn(*args, _stream(t))
+    if rc:
+        check(rc, what)
+
+
 def forward_project(geom: Geometry, vol: torch.Tensor, out: torch.Tensor | None = None,
                     accumulate: bool = False) -> torch.Tensor:
     """proj = P vol (or proj += P vol); vol [B, nz, ny, nx] -> proj [B, na, nv, nu]."""
@@ -109,14 +121,14 @@ def forward_project(geom: Geometry, vol: torch.Tensor, out: torch.Tensor | None 
     v = _batched(vol, geom.vol_shape, "forward_project")
     B = v.shape[0]
     if out is None:
-        out = torch.empty((B,) + geom.proj_shape, device=v.device, dtype=v.dtype)
+        o = out = torch.empty((B,) + geom.proj_shape, device=v.device, dtype=v.dtype)
         accumulate = False
-    o = out if out.dim() == 4 else out.unsqueeze(0)
-    assert o.is_contiguous() and o.dtype == v.dtype and tuple(o.shape) == (B,) + geom.proj_shape
+    else:
+        o = out if out.dim() == 4 else out.unsqueeze(0)
+        assert o.is_contiguous() and o.dtype == v.dtype and tuple(o.shape) == (B,) + geom.proj_shape
     lib = _lib.load()
     fn = lib.forward_project if v.dtype == torch.float32 else lib.forward_project_f64
-    with torch.cuda.device(v.device):
-        check(fn(geom.handle, _ptr(v), _ptr(o), B, int(accumulate), _stream(v)), "forward_project")
+    _run(fn, "forward_project", v, geom.handle, _ptr(v), _ptr(o), B, int(accumulate))
     return out[0] if (squeeze and out.dim() == 4) else out
 
 
@@ -127,14 +139,14 @@ def back_project(geom: Geometry, proj: torch.Tensor, out: torch.Tensor | None = 
     p = _batched(proj, geom.proj_shape, "back_project")
     B = p.shape[0]
     if out is None:
-        out = torch.empty((B,) + geom.vol_shape, device=p.device, dtype=p.dtype)
+        o = out = torch.empty((B,) + geom.vol_shape, device=p.device, dtype=p.dtype)
         accumulate = False
-    o = out if out.dim() == 4 else out.unsqueeze(0)
-    assert o.is_contiguous() and o.dtype == p.dtype and tuple(o.shape) == (B,) + geom.vol_shape
+    else:
+        o = out if out.dim() == 4 else out.unsqueeze(0)
+        assert o.is_contiguous() and o.dtype == p.dtype and tuple(o.shape) == (B,) + geom.vol_shape
     lib = _lib.load()
     fn = lib.back_project if p.dtype == torch.float32 else lib.back_project_f64
-    with torch.cuda.device(p.device):
-        check(fn(geom.handle, _ptr(p), _ptr(o), B, int(accumulate), _stream(p)), "back_project")
+    _run(fn, "back_project", p, geom.handle, _ptr(p), _ptr(o), B, int(accumulate))
     return out[0] if (squeeze and out.dim() == 4) else out
 
 
