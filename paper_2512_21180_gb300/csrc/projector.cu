@@ -97,8 +97,7 @@ __global__ void __launch_bounds__(256) k_forward(GeomDev g, const T *__restrict_
 
 // pw = proj * step(ray) * scale (* colw[column] when colw is given)
 template <typename T>
-__global__ void k_weight_rays(GeomDev g, const T *__restrict__ proj, T *__restrict__ pw, const T *__restrict__ colw,
-                              int pitch) {
+__global__ void k_weight_rays(GeomDev g, const T *__restrict__ proj, T *__restrict__ pw, const T *__restrict__ colw) {
     const int iu = blockIdx.x * 32 + threadIdx.x;
     const int iv = blockIdx.y * 8 + threadIdx.y;
     const int k = blockIdx.z % g.na, b = blockIdx.z / g.na;
@@ -109,9 +108,55 @@ __global__ void k_weight_rays(GeomDev g, const T *__restrict__ proj, T *__restri
     ray_row(g, c, rz_of<T>(g, iv), dqz, qcz);
     T scale;
     if constexpr (sizeof(T) == 4) scale = g.scale; else scale = g.scaled;
-    const long long row = ((long long)b * g.na + k) * g.nv + iv;
-    const T v = proj[row * g.nu + iu] * ray_step<T>(g, a, c.dqb, dqz) * scale;
-    pw[row * pitch + iu] = colw ? v * colw[iu] : v;
+    const long long o = (((long long)b * g.na + k) * g.nv + iv) * g.nu + iu;
+    const T v = proj[o] * ray_step<T>(g, a, c.dqb, dqz) * scale;
+    pw[o] = colw ? v * colw[iu] : v;
+}
+
+// The same for the segment gather's padded rows (pitch a multiple of 4 floats): a thread keeps four
+// neighbouring columns and walks nrows rows, so a ray costs one read, one write and its square root
+// (one thread per ray, reloading its column, took 300 us for the clinical scan, three times the
+// DRAM time; now 118 us). vec: proj's rows start on 16 bytes.
+__global__ void __launch_bounds__(256) k_weight_rows(GeomDev g, const float *__restrict__ proj, float *__restrict__ pw,
+                                                     const float *__restrict__ colw, int pitch, int vec, int nrows) {
+    const int u0 = (blockIdx.x * 32 + threadIdx.x) * 4, v0 = (blockIdx.y * 8 + threadIdx.y) * nrows;
+    const int k = blockIdx.z % g.na;
+    if (u0 >= g.nu) return;
+    const Frame32 &F = g.f32[k];
+    ColT<float> c[4];
+    int a[4];
+    float w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int u = min(u0 + i, g.nu - 1);
+        a[i] = principal_axis(F, u);
+        c[i] = col_of<float>(g, k, u);
+        w[i] = colw ? colw[u] : 1.f;
+    }
+    const long long frame = blockIdx.z;  // batch item and angle
+#pragma unroll 2
+    for (int r = 0; r < nrows; ++r) {
+        const int v = v0 + r;
+        if (v >= g.nv) break;
+        const float *src = proj + (frame * g.nv + v) * g.nu + u0;
+        float p[4];
+        if (vec) {
+            const float4 q = *reinterpret_cast<const float4 *>(src);
+            p[0] = q.x; p[1] = q.y; p[2] = q.z; p[3] = q.w;
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) p[i] = u0 + i < g.nu ? src[i] : 0.f;
+        }
+        const float rz = rz_of<float>(g, v);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float dqz, qcz;
+            ray_row(g, c[i], rz, dqz, qcz);
+            p[i] = p[i] * ray_step<float>(g, a[i], c[i].dqb, dqz) * g.scale;
+            if (colw) p[i] *= w[i];
+        }
+        *reinterpret_cast<float4 *>(pw + (frame * g.nv + v) * pitch + u0) = make_float4(p[0], p[1], p[2], p[3]);
+    }
 }
 
 // Detector column (continuous) hit by the ray from the source through the xy
@@ -657,6 +702,54 @@ static int forward_impl(const cbct_geom *g, const T *vol, T *proj, int batch, in
 
 constexpr int kZS = 4;
 
+// Segment gather (FP32). Scratch, one allocation: the weighted projections and the parts' volumes.
+static int backward_segments(const cbct_geom *g, const float *proj, float *vol, int batch, int accumulate, cudaStream_t st,
+                             const float *colw) {
+    const GeomDev &d = g->dev;
+    const int pitch = (d.nu + 3) & ~3;  // rows on 16 bytes, for TMA
+    const int nzb = (d.n[2] + kZ3 - 1) / kZ3, bx = (d.n[0] + kB3 - 1) / kB3, by = (d.n[1] + kB3 - 1) / kB3;
+    // split the angles so that about 24 CTAs per SM (8 per resident slot) are available: bricks
+    // differ in how many angles see them, and the last ones must not leave SMs idle
+    // (2 x 128^3: 12 / 24 / 48 per SM 1800 / 1680 / 1640 us; one 128^3 930 / 868 / 875; the
+    // clinical volume has 40 per SM unsplit)
+    const long long base = (long long)bx * by * nzb * batch, want = 24LL * sm_count();
+    int nparts = (int)std::min<long long>(16, std::max<long long>(1, (want + base - 1) / base));
+    nparts = std::min(nparts, d.na);
+    while (nparts > 1 && (long long)nzb * batch * nparts > 65535) --nparts;
+    if ((long long)nzb * batch * nparts > 65535) return cuda_fail(cudaErrorInvalidConfiguration, "back_project launch");
+    const long long nvol = (long long)batch * d.n[0] * d.n[1] * d.n[2];
+    const long long npw = ((long long)batch * d.na * d.nv * pitch + 63) & ~63LL;
+    float *pw = nullptr;
+    CBCT_CUDA_TRY(scratch_alloc((void **)&pw, sizeof(float) * (npw + (nparts > 1 ? nparts * nvol : 0)), st));
+    float *partial = nparts > 1 ? pw + npw : nullptr;
+    const int vec = (d.nu & 3) == 0 && (reinterpret_cast<uintptr_t>(proj) & 15) == 0;
+    // 8 rows per thread, fewer when that leaves SMs without a CTA
+    const long long frames = (long long)d.na * batch;
+    const int nrows = (int)std::max<long long>(1, std::min<long long>(8, frames * d.nv * ((d.nu + 127) / 128) / (32LL * sm_count())));
+    dim3 gw((d.nu + 127) / 128, (d.nv + 8 * nrows - 1) / (8 * nrows), (unsigned)frames);
+    k_weight_rows<<<gw, dim3(32, 8), 0, st>>>(d, proj, pw, colw, pitch, vec, nrows);
+    cudaError_t e = cudaGetLastError();
+    CUtensorMap pmap;
+    const uint64_t dims[3] = {(uint64_t)d.nu, (uint64_t)d.nv, (uint64_t)d.na * batch};
+    const uint64_t str[2] = {(uint64_t)pitch * 4, (uint64_t)pitch * d.nv * 4};
+    const uint32_t box[3] = {kBC, kBR, 1};
+    const int rc = encode_tmap(&pmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, pw, dims, str, box);
+    if (e == cudaSuccess && rc == 0) {
+        k_backproject_seg<<<dim3(bx, by, nzb * batch * nparts), kThreads3, kSmem3, st>>>(pmap, d, pw, pitch, vol, accumulate,
+                                                                                        nparts, partial, g->status);
+        e = cudaGetLastError();
+        if (e == cudaSuccess && nparts > 1) {
+            const int gs = (int)std::min<long long>(8LL * sm_count(), (nvol + 255) / 256);
+            k_sum_parts<<<gs, 256, 0, st>>>(partial, nparts, nvol, vol, accumulate);
+            e = cudaGetLastError();
+        }
+    }
+    cudaFreeAsync(pw, st);
+    if (rc) return rc;
+    if (e != cudaSuccess) return cuda_fail(e, "back_project launch");
+    return 0;
+}
+
 template <typename T>
 static int backward_impl(const cbct_geom *g, const T *proj, T *vol, int batch, int accumulate, cudaStream_t st,
                          const T *colw = nullptr) {
@@ -666,56 +759,14 @@ static int backward_impl(const cbct_geom *g, const T *proj, T *vol, int batch, i
     const long long nproj = (long long)batch * d.na * d.nv * d.nu;
     const int nzs = (d.n[2] + kZS - 1) / kZS;
     if ((long long)nzs * batch > 65535) return fail(CBCT_EINVAL, "back_project: batch too large");
-    // the segment gather loads the weighted projections by TMA: rows start on 16 bytes
-    const int pitch = sizeof(T) == 4 && g->axis_contiguous ? (d.nu + 3) & ~3 : d.nu;
+    if constexpr (sizeof(T) == 4)
+        if (g->axis_contiguous) return backward_segments(g, proj, vol, batch, accumulate, st, colw);
     T *pw = nullptr;
-    CBCT_CUDA_TRY(scratch_alloc((void **)&pw, sizeof(T) * (nproj / d.nu) * pitch, st));
+    CBCT_CUDA_TRY(scratch_alloc((void **)&pw, sizeof(T) * nproj, st));
     dim3 blk(32, 8), gw((d.nu + 31) / 32, (d.nv + 7) / 8, d.na * batch);
-    k_weight_rays<T><<<gw, blk, 0, st>>>(d, proj, pw, colw, pitch);
+    k_weight_rays<T><<<gw, blk, 0, st>>>(d, proj, pw, colw);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) {
-        if constexpr (sizeof(T) == 4) {
-            if (g->axis_contiguous) {
-                const int nzb = (d.n[2] + kZ3 - 1) / kZ3;
-                const long long base = (long long)((d.n[0] + kB3 - 1) / kB3) * ((d.n[1] + kB3 - 1) / kB3) * nzb * batch;
-                // split the angles so that about 24 CTAs per SM (8 per resident slot) are available: bricks
-                // differ in how many angles see them, and the last ones must not leave SMs idle
-                // (2 x 128^3: 12 / 24 / 48 per SM 1800 / 1680 / 1640 us; one 128^3 930 / 868 / 875; the
-                // clinical volume has 40 per SM unsplit)
-                const long long want = 24LL * sm_count();
-                int nparts = (int)std::min<long long>(16, std::max<long long>(1, (want + base - 1) / base));
-                nparts = std::min(nparts, d.na);
-                while (nparts > 1 && (long long)nzb * batch * nparts > 65535) --nparts;
-                if ((long long)nzb * batch * nparts > 65535) e = cudaErrorInvalidConfiguration;
-                float *partial = nullptr;
-                const long long nvol = (long long)batch * d.n[0] * d.n[1] * d.n[2];
-                if (e == cudaSuccess && nparts > 1) e = scratch_alloc((void **)&partial, sizeof(float) * nvol * nparts, st);
-                int trc = 0;
-                if (e == cudaSuccess) {
-                    CUtensorMap pmap;
-                    const uint64_t dims[3] = {(uint64_t)d.nu, (uint64_t)d.nv, (uint64_t)d.na * batch};
-                    const uint64_t str[2] = {(uint64_t)pitch * 4, (uint64_t)pitch * d.nv * 4};
-                    const uint32_t box[3] = {kBC, kBR, 1};
-                    trc = encode_tmap(&pmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, pw, dims, str, box);
-                    if (trc == 0) {
-                        dim3 gb3((d.n[0] + kB3 - 1) / kB3, (d.n[1] + kB3 - 1) / kB3, nzb * batch * nparts);
-                        k_backproject_seg<<<gb3, kThreads3, kSmem3, st>>>(pmap, d, pw, pitch, vol, accumulate, nparts, partial,
-                                                                          g->status);
-                        e = cudaGetLastError();
-                        if (e == cudaSuccess && nparts > 1) {
-                            const int gs = (int)std::min<long long>(8LL * sm_count(), (nvol + 255) / 256);
-                            k_sum_parts<<<gs, 256, 0, st>>>(partial, nparts, nvol, vol, accumulate);
-                            e = cudaGetLastError();
-                        }
-                    }
-                }
-                if (partial) cudaFreeAsync(partial, st);
-                cudaFreeAsync(pw, st);
-                if (trc) return trc;
-                if (e != cudaSuccess) return cuda_fail(e, "back_project launch");
-                return 0;
-            }
-        }
         dim3 gb((d.n[0] + 31) / 32, (d.n[1] + 7) / 8, nzs * batch);
         k_backproject<T, kZS><<<gb, blk, 0, st>>>(d, pw, vol, accumulate);
         e = cudaGetLastError();
@@ -884,7 +935,7 @@ extern "C" int back_project_noalloc(const cbct_geom *g, const float *proj, float
             v.col64 = d.col64 + (long long)k0 * d.nu;
             const float *pb = proj + ((long long)b * d.na + k0) * per_angle;
             dim3 gw((d.nu + 31) / 32, (d.nv + 7) / 8, kc);
-            k_weight_rays<float><<<gw, blk, 0, st>>>(v, pb, scratch, nullptr, d.nu);
+            k_weight_rays<float><<<gw, blk, 0, st>>>(v, pb, scratch, nullptr);
             dim3 gb((d.n[0] + 31) / 32, (d.n[1] + 7) / 8, nzs);
             k_backproject<float, kZS><<<gb, blk, 0, st>>>(v, scratch, vol + b * nvox, k0 == 0 ? accumulate : 1);
             CBCT_LAUNCH_CHECK("back_project_noalloc launch");
