@@ -266,7 +266,7 @@ __device__ __forceinline__ void tile_step(TileCoord &c, const TileCoord &st, int
 //  producer (warp 16, one lane): waits until the stage is free (empty[s]) and loads
 //    the item's NR input rows with one TMA box, completion counted on full[s]; an
 //    input plane outside the volume only arrives (its MMAs are skipped).
-//  MMA (warp 17, one lane): per tile picks TMEM accumulator j % nacc once the epilogue
+//  MMA (warp 17, the elected lane issues): per tile picks TMEM accumulator j % nacc once the epilogue
 //    has drained it (acce), waits for each item (full[s]), issues one 128 x N x 16
 //    MMA per (input row, column tap, pair of channel groups) or, for CG = 1, per
 //    (pair of input rows, column tap), commits the stage to
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(kWsThreads) k_conv_tc(const __grid_constant__ 
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sbias + NPAD);
     int *abort_flag = reinterpret_cast<int *>(tmem_slot + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     constexpr int kAcc = conv_nacc(kN);
     // warpgroup q's first tile is tile q: with fewer accumulators than warpgroups it would
     // wait on a barrier phase that has not started yet (a parity wait that passes at once)
@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(kWsThreads) k_conv_tc(const __grid_constant__ 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     const int ntw = (a.W + 127) / 128, nh = (a.H + RPT - 1) / RPT;
     const long long ntiles = (long long)a.nimg * a.D * nh * ntw;
@@ -374,7 +374,8 @@ __global__ void __launch_bounds__(kWsThreads) k_conv_tc(const __grid_constant__ 
             }
         }
     } else if (warp == kMmaWarp) {
-        if (lane == 0) {
+        {
+            const uint32_t leader = elect_leader();
             // column tap dw of input row r reads region r from pixel G - 1 + dw on
             const uint32_t rs16 = (uint32_t)(rs / 16);
             const uint64_t adesc0 = smem_desc_kmajor(sA_u + (uint32_t)((a.G - 1) * 16), rs, 128);
@@ -389,6 +390,7 @@ __global__ void __launch_bounds__(kWsThreads) k_conv_tc(const __grid_constant__ 
                     *abort_flag = 1;
                     break;
                 }
+                __syncwarp();
                 tc_fence_after();
                 const uint32_t dt = tmem + (uint32_t)(ab * kN);
                 uint32_t acc_flag = 0;  // the tile's first MMA overwrites the accumulator
@@ -397,6 +399,7 @@ __global__ void __launch_bounds__(kWsThreads) k_conv_tc(const __grid_constant__ 
                         *abort_flag = 1;
                         break;
                     }
+                    __syncwarp();
                     const int d2 = tc.d + (nch == 3 ? c - 1 : 0);
                     if (d2 >= 0 && d2 < a.D) {
                         tc_fence_after();
@@ -419,7 +422,7 @@ __global__ void __launch_bounds__(kWsThreads) k_conv_tc(const __grid_constant__ 
                                 for (int dw = 0; dw < 3; ++dw) {
                                     const uint32_t ao = (uint32_t)(2 * j) * rs16 + (uint32_t)dw;
                                     const uint32_t bo = (uint32_t)((dw * 2 * nj * 16) >> 4);
-                                    mma_bf16(dtj, ad + ao, bd + bo, idesc, acc);
+                                    mma_bf16(dtj, ad + ao, bd + bo, idesc, acc, leader);
                                     acc = 1u;
                                 }
                             } else {
@@ -429,21 +432,21 @@ __global__ void __launch_bounds__(kWsThreads) k_conv_tc(const __grid_constant__ 
                                     for (int kp = 0; kp < kCGP; kp += 2) {
                                         const uint32_t ao = (uint32_t)(j * CG + kp) * rs16 + (uint32_t)dw;
                                         const uint32_t bo = (uint32_t)(((dw * kCGP + kp) * nj * 16) >> 4);
-                                        mma_bf16(dtj, ad + ao, bd + bo, idesc, acc);
+                                        mma_bf16(dtj, ad + ao, bd + bo, idesc, acc, leader);
                                         acc = 1u;
                                     }
                             }
                         }
                         acc_flag = 1u;
                     }
-                    mma_commit(&empty[s]);
+                    mma_commit(&empty[s], leader);
                     if (++s == nst) {
                         s = 0;
                         ph ^= 1u;
                     }
                 }
                 if (*abort_flag) break;
-                mma_commit(&accf[ab]);
+                mma_commit(&accf[ab], leader);
                 tile_next(tc, a.D, nh, a.W);
             }
         }
@@ -586,7 +589,7 @@ __global__ void k_pack_jobs(const ConvPackJob *__restrict__ jobs, const float *_
 // 2048 B) accumulates D_dw[(r, ci)][(o, co)] in TMEM over every tile of the CTA. Entry
 // (r, o) belongs to tap dh = r - 1 - o: six of the eight (r, o) pairs are taps, and two
 // pairs (o = 0, 1) give each tap: the epilogue adds them through shared memory, each CTA writes
-// one partial of its 9 taps and a fixed-order reduction adds the CTAs (deterministic). Two dY rows
+// partials of its 9 taps and a fixed-order reduction adds them (deterministic). Two dY rows
 // per MMA halve the MMA count per output row, and the three taps dd in separate CTAs keep the
 // accumulators at 3 x N <= 192 TMEM columns, so two CTAs (two MMA issuers) share an SM.
 // The bias gradient is summed by the epilogue warps of the middle depth tap's CTAs from the dY
@@ -605,13 +608,14 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32_mn(int M, int N) {
 // groups per dY row: 2 (16 outputs, the second group zero when cout <= 8) or 4.
 // Grid: ndd x gpd CTAs, the depth taps of a range of tiles next to each other: they run at the
 // same time on the same planes, and the tiles of a CTA are gpd apart, so that all CTAs move through the
-// planes together and read them from L2 (at 128^3 x 32 channels: 268 MB and 127 us, the MMAs now the limit; with the taps as three successive
-// waves every plane came from DRAM three times, 813 MB, 78 % of the DRAM rate).
-// partial: [ndd][gpd][cout][9][cin]; partial_b (null without a bias): [gpd][cout].
+// planes together and read them from DRAM once (at 128^3 x 32 channels 268 MB; with the taps as three
+// successive waves 813 MB, 78 % of the DRAM rate).
+// partial: [ndd][gpd][nseg][cout][9][cin], one per segment of the CTA's tiles; partial_b (null without a
+// bias): [gpd][cout].
 template <int XCG, int NCG>
 __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_constant__ CUtensorMap xmap,
                                                               const __grid_constant__ CUtensorMap ymap, ConvArgs a,
-                                                              int cgo, float *__restrict__ partial,
+                                                              int cgo, int nseg, float *__restrict__ partial,
                                                               float *__restrict__ partial_b) {
     constexpr int kN = 2 * NCG * 8;
     constexpr int kYBytes = 2 * NCG * 2048;
@@ -621,15 +625,15 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
     unsigned char *sm = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     uint64_t *full = reinterpret_cast<uint64_t *>(sm + kWgStages * kStage);
     uint64_t *empty = full + kWgStages;
-    uint64_t *done = empty + kWgStages;
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 1);
+    uint64_t *done = empty + kWgStages, *drained = done + 1;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drained + 1);
     int *abort_flag = reinterpret_cast<int *>(tmem_slot + 1);
-    int *used = abort_flag + 1;  // [3]: accumulator dw received an MMA
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    int *used = abort_flag + 1;  // [3]: accumulator dw received an MMA in this segment
+    float *xch = reinterpret_cast<float *>(used + 3);  // [3][16][32]: tap sums on their way between warps
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int ndd = a.taps3d ? 3 : 1, gpd = (int)gridDim.x / ndd;
     const int dd = blockIdx.x % ndd, cta = blockIdx.x / ndd;  // depth tap (3-D: input plane d + dd - 1), its CTA
     const bool bias = partial_b && dd == (a.taps3d ? 1 : 0);  // (the middle tap's input plane always exists)
-    static_assert(9 * 32 * 32 * sizeof(float) <= kWgStages * (kWgXBytes + 2 * 2 * 2048), "tap sums in the stages");
     constexpr uint32_t kIdesc = idesc_bf16_f32_mn(128, kN);
     const int rs = 16 * a.G * conv_box_rows(a.G);
 
@@ -639,7 +643,8 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], bias ? 5 : 1);  // the MMAs' commit (and the four epilogue warps)
         }
-        mbar_init(done, 2);  // the MMAs' commit + the MMA thread's release of used[]
+        mbar_init(done, 2);     // a segment's MMAs: their commit + the MMA thread's release of used[]
+        mbar_init(drained, 4);  // its accumulators read by the four epilogue warps
         *abort_flag = 0;
         for (int i = 0; i < 3; ++i) used[i] = 0;
         fence_mbar_init();
@@ -666,13 +671,14 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     const int ntw = (a.W + 127) / 128, nh = (a.H + 1) / 2;
     const long long ntiles = (long long)a.nimg * a.D * nh * ntw;
     // tiles cta, cta + gpd, ...: the CTAs move through the planes together
     const long long t_begin = cta, my_tiles = cta < ntiles ? (ntiles - cta + gpd - 1) / gpd : 0;
     const TileCoord step = tile_coord(gpd, a.D, nh, ntw);
+    auto seg_end = [&](int seg) { return my_tiles * (seg + 1) / nseg; };  // tiles of segments 0 .. seg
     const uint32_t sm_u = smem_u32(sm);
 
     if (warp == 4) {
@@ -715,16 +721,40 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
             }
         }
     } else if (warp == 5) {
-        if (lane == 0) {
+        {
+            const uint32_t leader = elect_leader();
             TileCoord tc = tile_coord(t_begin, a.D, nh, ntw);
             int s = 0;
             uint32_t ph = 0;
             uint32_t usedm = 0;  // bit dw: accumulator initialised
+            int seg = 0;
+            // the segment's accumulators to the epilogue (a segment without MMAs, in a CTA without
+            // tiles, arrives directly instead of committing)
+            auto hand_over = [&]() {
+                __syncwarp();
+                if (leader)
+                    for (int k = 0; k < 3; ++k) used[k] = (usedm >> k) & 1u;
+                if (usedm) mma_commit(done, leader);
+                else if (leader) mbar_arrive(done);
+                if (leader) mbar_arrive(done);
+                usedm = 0;
+                ++seg;
+            };
             for (long long i = 0; i < my_tiles && !*abort_flag; ++i) {
-                if (!mbar_wait(&full[s], ph, a.status)) {
+                while (i == seg_end(seg)) {
+                    hand_over();
+                    if (!mbar_wait(drained, (uint32_t)((seg - 1) & 1), a.status)) {
+                        *abort_flag = 1;
+                        break;
+                    }
+                    __syncwarp();
+                    tc_fence_after();
+                }
+                if (*abort_flag || !mbar_wait(&full[s], ph, a.status)) {
                     *abort_flag = 1;
                     break;
                 }
+                __syncwarp();
                 const int d2 = tc.d + (a.taps3d ? dd - 1 : 0);
                 if (d2 >= 0 && d2 < a.D) {
                     tc_fence_after();
@@ -738,33 +768,32 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
                             // pixels = 128 B), the stride byte offset along M / N
                             const uint64_t ad = smem_desc_kmajor(st + (uint32_t)((a.G - 1 + dw) * 16 + ks * 256), 128, rs);
                             const uint64_t bd = smem_desc_kmajor(st + kWgXBytes + (uint32_t)(ks * 256), 128, 2048);
-                            mma_bf16(dt, ad, bd, kIdesc, (usedm >> dw) & 1u);
+                            mma_bf16(dt, ad, bd, kIdesc, (usedm >> dw) & 1u, leader);
                             usedm |= 1u << dw;
                         }
                     }
                 }
-                mma_commit(&empty[s]);
+                mma_commit(&empty[s], leader);
                 tile_step(tc, step, a.D, nh, ntw);
                 if (++s == kWgStages) {
                     s = 0;
                     ph ^= 1u;
                 }
             }
-            for (int k = 0; k < 3; ++k) used[k] = (usedm >> k) & 1u;
-            // a CTA without tiles (the last ones when the tiles do not divide evenly) issued
-            // no MMA: it arrives directly instead of committing
-            if (usedm) mma_commit(done);
-            else mbar_arrive(done);
-            mbar_arrive(done);
+            hand_over();
+            for (; seg < nseg;) {  // (segments past the tiles of a CTA with few)
+                if (!mbar_wait(drained, (uint32_t)((seg - 1) & 1), a.status)) break;
+                hand_over();
+            }
         }
     } else {
-        if (bias) {
-            // warp = output-channel group, lane = pixels lane, lane + 32, ... of both dY rows (zero
-            // outside the image)
-            float sum[8] = {};
-            int s = 0;
-            uint32_t ph = 0;
-            for (long long i = 0; i < my_tiles; ++i) {
+        float sum[8] = {};  // bias: warp = output-channel group, lane = pixels lane, lane + 32, ...
+        int s = 0;
+        uint32_t ph = 0;
+        long long i = 0;
+        for (int seg = 0; seg < nseg; ++seg) {
+            for (; bias && i < seg_end(seg); ++i) {
+                // the lane's pixels of both dY rows (zero outside the image)
                 if (!mbar_wait(&full[s], ph, a.status)) {
                     *abort_flag = 1;
                     break;
@@ -790,51 +819,49 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
                     ph ^= 1u;
                 }
             }
+            // warp w holds accumulator rows 32 w .. 32 w + 31 = input row r = w, input channel = lane;
+            // columns (o, co). Pair (r, o) is tap dh = r - 1 - o: row r's o = 1 columns go through
+            // shared memory to row r - 1's o = 0 ones, 16 columns at a time
+            const bool ok = mbar_wait(done, (uint32_t)(seg & 1), a.status) && !*abort_flag;
+            tc_fence_after();
+            float *pb = partial + (((long long)dd * gpd + cta) * nseg + seg) * a.cout * 9 * a.cin;
+#pragma unroll 1
+            for (int dw = 0; dw < 3; ++dw) {
+                const bool valid = ok && used[dw];
+#pragma unroll 1
+                for (int c0 = 0; c0 < NCG * 8; c0 += 16) {
+                    float v[16];
+                    const uint32_t t = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(dw * kN + c0);
+                    if (warp >= 1) {
+                        tmem_ld16(t + NCG * 8, v);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) xch[((warp - 1) * 16 + j) * 32 + lane] = v[j];
+                    }
+                    asm volatile("bar.sync 1, 128;" ::: "memory");  // the four epilogue warps
+                    if (warp < 3) {
+                        tmem_ld16(t, v);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            const int co = c0 + j;
+                            const float x = xch[(warp * 16 + j) * 32 + lane];
+                            if (lane < a.cin && co < a.cout)
+                                pb[((long long)co * 9 + warp * 3 + dw) * a.cin + lane] = valid ? v[j] + x : 0.f;
+                        }
+                    }
+                    asm volatile("bar.sync 1, 128;" ::: "memory");
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(drained);
+        }
+        if (bias) {
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) sum[j] += __shfl_xor_sync(0xffffffffu, sum[j], o);
                 const int co = 8 * warp + j;
                 if (lane == 0 && warp < cgo && co < a.cout) partial_b[(long long)cta * a.cout + co] = sum[j];
-            }
-        }
-        // epilogue (warps 0-3): warp w holds accumulator rows 32 w .. 32 w + 31 = input
-        // row r = w, input channel = lane; columns (o, co). Pair (r, o) is tap dh = r - 1 - o: row r's
-        // o = 1 columns go through shared memory (the stages are free) to row r - 1's o = 0 ones
-        const bool ok = mbar_wait(done, 0u, a.status);
-        tc_fence_after();
-        float *tap = reinterpret_cast<float *>(sm);  // [dw][dh + 1][co][32]
-        constexpr int kTap = NCG * 8 * 32;
-        const long long per_o = (long long)a.cout * 9 * a.cin;
-        float *pb = partial + ((long long)dd * gpd + cta) * per_o;
-        if (warp >= 1) {
-#pragma unroll 1
-            for (int dw = 0; dw < 3; ++dw)
-#pragma unroll
-                for (int c0 = 0; c0 < NCG * 8; c0 += 16) {
-                    float v[16];
-                    tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(dw * kN + NCG * 8 + c0), v);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) tap[(dw * 3 + warp - 1) * kTap + (c0 + j) * 32 + lane] = v[j];
-                }
-        }
-        asm volatile("bar.sync 1, 128;" ::: "memory");  // the four epilogue warps
-        if (warp < 3) {
-#pragma unroll 1
-            for (int dw = 0; dw < 3; ++dw) {
-                const bool valid = ok && !*abort_flag && used[dw];
-#pragma unroll
-                for (int c0 = 0; c0 < NCG * 8; c0 += 16) {
-                    float v[16];
-                    tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(dw * kN + c0), v);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int co = c0 + j;
-                        if (lane < a.cin && co < a.cout)
-                            pb[((long long)co * 9 + warp * 3 + dw) * a.cin + lane] =
-                                valid ? v[j] + tap[(dw * 3 + warp) * kTap + co * 32 + lane] : 0.f;
-                    }
-                }
             }
         }
     }
@@ -847,11 +874,11 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
 }
 
 // out[co0 + co][tap][ci0 + ci] (+)= sum over the CTAs of their tap's partials, fixed order: partial
-// [ndd][gpd][cout][9][cin], tap = dd * 9 + t9; out has cin_full input channels per tap. The
+// [ndd][gpd nseg][cout][9][cin], tap = dd * 9 + t9; out has cin_full input channels per tap. The
 // blocks past the weights' sum the bias partials partial_b [gpd][cout] into db. A block takes 32
 // sums, each as 8 slices of the CTAs added in order: enough loads in flight to read the partials at L2
 // speed (one thread per sum took 65 us for 67 MB; now 10 us for 34 MB).
-__global__ void __launch_bounds__(256) k_reduce_wgrad(const float *__restrict__ partial, int gpd, int ndd, int cout, int cin,
+__global__ void __launch_bounds__(256) k_reduce_wgrad(const float *__restrict__ partial, int gpd, int nseg, int ndd, int cout, int cin,
                                                       float *__restrict__ out, int accumulate, int co0, int ci0, int cin_full,
                                                       const float *__restrict__ partial_b, float *__restrict__ db) {
     __shared__ float red[8][32];
@@ -862,12 +889,13 @@ __global__ void __launch_bounds__(256) k_reduce_wgrad(const float *__restrict__ 
     const bool ok = i < (is_b ? cout : n);
     const int ci = i % cin, tap = (i / cin) % (9 * ndd), co = i / (cin * 9 * ndd), d = tap / 9, t9 = tap % 9;
     const long long stride = is_b ? cout : (long long)cout * 9 * cin;
-    const float *p = is_b ? partial_b + i : partial + (long long)d * gpd * stride + ((long long)co * 9 + t9) * cin + ci;
+    const float *p = is_b ? partial_b + i : partial + (long long)d * gpd * nseg * stride + ((long long)co * 9 + t9) * cin + ci;
+    const int np = is_b ? gpd : gpd * nseg;
     float s = 0.f;
     if (ok) {
-        const int b1 = gpd * (sl + 1) / 8;
+        const int b1 = np * (sl + 1) / 8;
 #pragma unroll 8
-        for (int b = gpd * sl / 8; b < b1; ++b) s += p[b * stride];
+        for (int b = np * sl / 8; b < b1; ++b) s += p[b * stride];
     }
     red[sl][lane] = s;
     __syncthreads();
@@ -1117,19 +1145,22 @@ static int conv_wgrad_tc(const __nv_bfloat16 *x, int xgs, int cin, const __nv_bf
         if (rc) return rc;
     }
     constexpr size_t kStage = kWgXBytes + 2 * NCG * 2048;
-    const size_t smem = 1024 + kWgStages * kStage + 8 * (2 * kWgStages + 1) + 4 * 5 + 64;
+    const size_t smem = 1024 + kWgStages * kStage + 8 * (2 * kWgStages + 2) + 4 * 5 + 3 * 16 * 32 * 4 + 64;
     CBCT_CUDA_TRY(cudaFuncSetAttribute(k_conv_wgrad_tc<XCG, NCG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int nsm = sm_count();
     const int ndd = taps3d ? 3 : 1;
     const long long ntiles = (long long)nimg * D * ((H + 1) / 2) * ((W + 127) / 128);
-    const int gpd = (int)std::max<long long>(1, std::min<long long>(ntiles, 2LL * nsm / ndd));  // CTAs per depth tap
+    // CTAs per depth tap: as many as run at the same time (two per SM over all taps). Each writes a partial
+    // per segment of its tiles: one accumulation in TMEM over all of a 3-D layer's tiles would more than double
+    // the error against 64 bits (128^3: 4.0e-6 with 27 tiles, 9.3e-6 with 81)
+    const int gpd = (int)std::max<long long>(1, std::min<long long>(ntiles, 2LL * nsm / ndd)), nseg = ndd;
     const long long per_cta = (long long)cout * 9 * cin;
     const int nw = cout * 9 * ndd * cin;
     float *part = nullptr;
-    CBCT_CUDA_TRY(scratch_alloc((void **)&part, sizeof(float) * ((long long)ndd * gpd * per_cta + (long long)gpd * cout), st));
-    float *partb = db ? part + (long long)ndd * gpd * per_cta : nullptr;
-    k_conv_wgrad_tc<XCG, NCG><<<gpd * ndd, kWgThreads, smem, st>>>(xmap, ymap, a, cgo, part, partb);
-    k_reduce_wgrad<<<(nw + 31) / 32 + (db ? (cout + 31) / 32 : 0), 256, 0, st>>>(part, gpd, ndd, cout, cin, dw, accumulate, co0,
+    CBCT_CUDA_TRY(scratch_alloc((void **)&part, sizeof(float) * ((long long)ndd * gpd * nseg * per_cta + (long long)gpd * cout), st));
+    float *partb = db ? part + (long long)ndd * gpd * nseg * per_cta : nullptr;
+    k_conv_wgrad_tc<XCG, NCG><<<gpd * ndd, kWgThreads, smem, st>>>(xmap, ymap, a, cgo, nseg, part, partb);
+    k_reduce_wgrad<<<(nw + 31) / 32 + (db ? (cout + 31) / 32 : 0), 256, 0, st>>>(part, gpd, nseg, ndd, cout, cin, dw, accumulate, co0,
                                                                                ci0, cin_full, partb, db);
     cudaError_t e = cudaGetLastError();
     cudaFreeAsync(part, st);
