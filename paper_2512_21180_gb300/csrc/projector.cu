@@ -714,6 +714,11 @@ static int backward_segments(const cbct_geom *g, const float *proj, float *vol, 
     // clinical volume has 40 per SM unsplit)
     const long long base = (long long)bx * by * nzb * batch, want = 24LL * sm_count();
     int nparts = (int)std::min<long long>(16, std::max<long long>(1, (want + base - 1) / base));
+    // parts of at least 8 angles, as long as that leaves two waves of 3 CTAs per SM: a CTA's set-up
+    // and its write and re-read of a partial volume cost about as much as two angles (64^3 at 4 mm:
+    // 64 angles 58.5 -> 54.0 us, two volumes 107.7 -> 92.3, 32 angles 43.7 -> 36.3; 100^3, 40 angles
+    // 80.1 -> 76.7; with one wave 40.7 and 16 angles 68 at 64 and 32 angles, with four no change)
+    nparts = (int)std::min<long long>(nparts, std::max<long long>((d.na + 7) / 8, (6LL * sm_count() + base - 1) / base));
     nparts = std::min(nparts, d.na);
     while (nparts > 1 && (long long)nzb * batch * nparts > 65535) --nparts;
     if ((long long)nzb * batch * nparts > 65535) return cuda_fail(cudaErrorInvalidConfiguration, "back_project launch");

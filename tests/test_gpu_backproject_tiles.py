@@ -17,6 +17,8 @@ CASES = {
     "fine_panel": I.scaled(T, n=(20, 18, 11), vox=(8.0, 8.0, 8.0), nu=601, nv=333, du=0.41, dv=0.43, n_angles=3),
     # one part of more than 128 angles (16 parts)
     "many_angles": I.scaled(T, n=(17, 16, 9), n_angles=2100),
+    # 64 bricks and more: parts of eight angles and a last one of fewer
+    "eight_per_part": I.scaled(T, n=(64, 52, 60), vox=(4.0, 4.0, 4.0), nu=90, nv=60, du=2.9, dv=4.1, n_angles=61),
     # panels of one row, one column, and widths around a multiple of 4
     "one_row": I.scaled(T, nv=1, nu=31, n_angles=5),
     "one_column": I.scaled(T, nu=1, nv=29, n_angles=5),
