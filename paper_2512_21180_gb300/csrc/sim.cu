@@ -154,19 +154,20 @@ __global__ void k_water_bone(const float *__restrict__ mu, long long nvox, long 
 // once. With FP64 draws the kernel was bound by the FP64 pipe (83 % of it); the draws of
 // poisson.cuh decide all but 1e-4 of them in FP32. 9.8 M pixels x 10 bins (CUDA events): 66.7 ms ->
 // 2.4 ms (41 G draws/s).
-__global__ void __launch_bounds__(256) k_poly_reading(const float *__restrict__ L, int frames_per_item, int nframes,
-                                                      int npix, int group, const float *__restrict__ I0, PolyTab t,
+__global__ void __launch_bounds__(256) k_poly_reading(const float *__restrict__ L, long long frames_per_item,
+                                                      long long nframes, int npix, long long group, const float *__restrict__ I0, PolyTab t,
                                                       unsigned long long seed, int noise, float *__restrict__ reading,
                                                       float *__restrict__ y, int32_t *__restrict__ counts) {
     const int pix = blockIdx.x * blockDim.x + threadIdx.x;
     if (pix >= npix) return;
-    const int f0 = blockIdx.y * group, f1 = min(f0 + group, nframes);
+    const long long f0 = blockIdx.y * group, f1 = min(f0 + group, nframes);
     double air = 0.0;
     for (int j = 0; j < t.ne; ++j) air = __dadd_rn(air, __dmul_rn(t.resp[j], (double)I0[(long long)j * npix + pix]));
     const long long per_item = (long long)frames_per_item * npix;
-    for (int f = f0; f < f1; ++f) {
-        const int b = f / frames_per_item;
-        const long long e = (long long)f * npix + pix, w = e + b * per_item;  // water; bone one item on
+    long long b = f0 / frames_per_item, left = (b + 1) * frames_per_item - f0;  // item, its frames to go
+    for (long long f = f0; f < f1; ++f) {
+        if (left-- == 0) ++b, left = frames_per_item - 1;
+        const long long e = f * npix + pix, w = e + b * per_item;  // water; bone one item on
         const float Lw = L[w], Lb = L[w + per_item];
         double acc = 0.0;
         for (int j = 0; j < t.ne; ++j) {
@@ -278,12 +279,11 @@ __global__ void k_fov(GeomDev g, const double *__restrict__ cs, double sid, doub
 static int poly_launch(const float *L, int batch, long long n_per_item, int npix, const float *I0, const PolyTab &t,
                        unsigned long long seed, int noise, float *reading, float *y, int32_t *counts, cudaStream_t st) {
     const long long frames_per_item = n_per_item / npix, nframes = frames_per_item * batch;
-    if (nframes > 0x7fffffffLL) return fail(CBCT_EINVAL, "cbct_poly_reading: too many frames");
     long long group = nframes * npix / (4LL * 2048 * sm_count());
     group = group < 1 ? 1 : group > 16 ? 16 : group;
     if ((nframes + group - 1) / group > 65535) group = (nframes + 65534) / 65535;
     dim3 grd((unsigned)((npix + 255) / 256), (unsigned)((nframes + group - 1) / group));
-    k_poly_reading<<<grd, 256, 0, st>>>(L, (int)frames_per_item, (int)nframes, npix, (int)group, I0, t, seed, noise ? 1 : 0,
+    k_poly_reading<<<grd, 256, 0, st>>>(L, frames_per_item, nframes, npix, group, I0, t, seed, noise ? 1 : 0,
                                         reading, y, counts);
     CBCT_LAUNCH_CHECK("cbct_poly_reading launch");
     return 0;
