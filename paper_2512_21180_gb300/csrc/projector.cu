@@ -273,21 +273,23 @@ __global__ void __launch_bounds__(256) k_backproject(GeomDev g, const T *__restr
 // so the tile of the projection that the brick sees at one angle is loaded once (TMA, the
 // next tile in flight while this one is summed), turned into prefix sums (sum p,
 // sum (row - h) p) down each column, and every interval is the difference of two entries:
-// 12 instructions instead of a run of predicated row loads (3 to 5 rows per interval at
-// these magnifications). The sums start at the tile's middle row h and run outwards, so
+// 10 instructions instead of a run of predicated row loads (3 to 5 rows per interval at
+// these magnifications); boundaries, shares and sums of two voxels go through packed FP32
+// instructions (12, one voxel at a time, with the same results: clinical 9.02 against 8.82 ms). The sums start at the tile's middle row h and run outwards, so
 // they span at most half a tile (26 rows) of one column: FP32 rounding stays that of a
 // short sum, and the measured error against 64 bits is the row-by-row kernel's (clinical
-// 3.5e-7 both). Bounded by instruction issue: about 3/4 of the instructions are the
-// intervals, 1/8 the prefix sums. Back projection by CUDA events, before -> after:
-// clinical 17.4 -> 9.3 ms, 2 x 128^3 / 200 angles 3.79 -> 1.68 ms, 181 x 167 x 93 / 150 angles
-// 4.12 -> 1.26 ms, 64^3 / 64 angles 126 -> 69 us.
+// 3.3e-7 against 3.5e-7). Bounded by instruction issue (62 % of the issue slots; the rest
+// mostly the two barriers of a tile, 24 % of the stalls): about 3/4 of the instructions are the
+// intervals, 1/8 the prefix sums. Back projection by CUDA events, row by row -> now:
+// clinical 17.4 -> 8.82 ms, 2 x 128^3 / 200 angles 3.79 -> 1.58 ms, 181 x 167 x 93 / 150 angles
+// 4.12 -> 1.19 ms, 64^3 / 64 angles 126 -> 60 us.
 //
 // A tile whose sums are not finite (an infinite or NaN pixel, or an overflow) is summed row
 // by row instead, so such a pixel reaches the voxels its ray touches and no others. A brick
 // whose footprint exceeds the tile takes several tiles per angle: the intervals are linear in
 // the rows, so a tile that holds part of an interval adds its part.
 //
-// Tile 112 x 52: the largest that lets three CTAs share an SM (clinical 9.3 ms; 96 x 60 9.7,
+// Tile 112 x 52: the largest that lets three CTAs share an SM (clinical, one voxel at a time, 9.3 ms; 96 x 60 9.7,
 // 120 x 48 9.8, 128 x 46 10.0, 80 x 64 11.0 with more tiles split in columns; 112 x 56 at two
 // CTAs per SM 10.9; without the TMA stage, reading the rows from L2, 10.6 at three and 12.5
 // at four CTAs of 56 registers).
@@ -349,9 +351,9 @@ __global__ void __launch_bounds__(kThreads3, 3)
         const int i = i0 + il, s = j0 - 1 + seg;
         const bool mine = item && i < g.n[a] && s < g.n[1 - a];
         const float di = (float)i - 0.5f * (float)(g.n[a] - 1);
-        float SA[kZ3], SB[kZ3];
+        float2 SA[kZ3 / 2], SB[kZ3 / 2];  // two voxels each
 #pragma unroll
-        for (int m = 0; m < kZ3; ++m) SA[m] = SB[m] = 0.f;
+        for (int q = 0; q < kZ3 / 2; ++q) SA[q] = SB[q] = make_float2(0.f, 0.f);
 #pragma unroll 1
         for (int kc = k_begin; kc < k_end; kc += kChunk3) {
             // list the angles of this chunk that reach the brick, in order
@@ -521,26 +523,38 @@ __global__ void __launch_bounds__(kThreads3, 3)
                             // is floor(x). In units of step, the rows of interval m weigh
                             // S1 = T - (x - 1 - h) S0 on the upper voxel and irs S0 - S1 on the lower.
                             const float h1 = (float)(h + 1), vb = fmaf(-qh, irs, h1);
-                            const float sl = wl * step, su = wu * step;
+                            const float2 irs2 = make_float2(irs, irs), vb2 = make_float2(vb, vb), h12 = make_float2(h1, h1);
+                            const float2 sl2 = make_float2(wl * step, wl * step), su2 = make_float2(wu * step, wu * step);
                             const float2 *Eu = E + (u - u0);
-                            auto above = [&](float x) { return Eu[min(__float2uint_rd(x), (unsigned)nr) * (unsigned)kEP]; };
-                            float x = vb, carry = 0.f;  // upper-voxel share of the previous interval
-                            float2 e = above(x);
-#pragma unroll
-                            for (int m = 0; m < kZ3 + 1; ++m) {
-                                const float xn = fmaf((float)(m + 1), irs, vb);
-                                const float2 f = above(xn);
+                            auto rows = [&](float2 &e, float x) {  // sums between the last boundary and x
+                                const float2 f = Eu[min(__float2uint_rd(x), (unsigned)nr) * (unsigned)kEP];
                                 const float2 d = __fadd2_rn(f, make_float2(-e.x, -e.y));
-                                const float S1 = fmaf(h1 - x, d.x, d.y);
-                                // voxel z0 - 1 + m: upper share of interval m - 1, lower share of interval m
-                                if (m >= 1) {
-                                    const float R = carry + fmaf(irs, d.x, -S1);
-                                    SA[m - 1] = fmaf(sl, R, SA[m - 1]);
-                                    SB[m - 1] = fmaf(su, R, SB[m - 1]);
-                                }
-                                carry = S1;
                                 e = f;
-                                x = xn;
+                                return d;
+                            };
+                            // boundary m's x and h + 1 - x, two at a time
+                            auto ends = [&](float m, float2 &x, float2 &y) {
+                                x = __ffma2_rn(make_float2(m, m + 1.f), irs2, vb2);
+                                y = __fadd2_rn(h12, make_float2(-x.x, -x.y));
+                            };
+                            float2 x, y, e = make_float2(0.f, 0.f);
+                            ends(0.f, x, y);
+                            rows(e, x.x);
+                            float2 d = rows(e, x.y);
+                            float carry = fmaf(y.x, d.x, d.y);  // upper-voxel share of the previous interval
+#pragma unroll
+                            for (int q = 0; q < kZ3 / 2; ++q) {
+                                // voxels z0 + 2 q and z0 + 2 q + 1: upper share of interval m - 1, lower share of m
+                                float2 xn, yn;
+                                ends(2.f * q + 2.f, xn, yn);
+                                const float2 d1 = rows(e, xn.x), d2 = rows(e, xn.y);
+                                const float s1 = fmaf(y.y, d1.x, d1.y), s2 = fmaf(yn.x, d2.x, d2.y);
+                                const float2 R = __fadd2_rn(make_float2(carry, s1), make_float2(fmaf(irs, d1.x, -s1),
+                                                                                                fmaf(irs, d2.x, -s2)));
+                                SA[q] = __ffma2_rn(sl2, R, SA[q]);
+                                SB[q] = __ffma2_rn(su2, R, SB[q]);
+                                carry = s2;
+                                y = yn;
                             }
                         } else {
                             const float *Pu = pw + ((long long)(b * g.na + k) * nv + v0) * pitch + u;
@@ -549,11 +563,12 @@ __global__ void __launch_bounds__(kThreads3, 3)
                                 const float p = __ldg(Pu + (long long)r * pitch);
                                 const float q = fmaf((float)(r - h), step, qh);
 #pragma unroll
-                                for (int m = 1; m <= kZ3; ++m) {
-                                    const float w = 1.0f - fabsf(q - (float)m);
+                                for (int m = 0; m < kZ3; ++m) {
+                                    const float w = 1.0f - fabsf(q - (float)(m + 1));
+                                    float &sa = m & 1 ? SA[m / 2].y : SA[m / 2].x, &sb = m & 1 ? SB[m / 2].y : SB[m / 2].x;
                                     if (w > 0.f) {
-                                        SA[m - 1] = fmaf(wl, w * p, SA[m - 1]);
-                                        SB[m - 1] = fmaf(wu, w * p, SB[m - 1]);
+                                        sa = fmaf(wl, w * p, sa);
+                                        sb = fmaf(wu, w * p, sb);
                                     }
                                 }
                             }
@@ -580,13 +595,13 @@ __global__ void __launch_bounds__(kThreads3, 3)
             const int vl = seg - 1;
             float *v = vacc + (a == 0 ? vl * (kB3 + 1) + il : il * (kB3 + 1) + vl);
 #pragma unroll
-            for (int m = 0; m < kZ3; ++m) v[m * kB3 * (kB3 + 1)] += SA[m];
+            for (int m = 0; m < kZ3; ++m) v[m * kB3 * (kB3 + 1)] += m & 1 ? SA[m / 2].y : SA[m / 2].x;
         }
         __syncthreads();
         if (mine && seg < kB3) {
             float *v = vacc + (a == 0 ? seg * (kB3 + 1) + il : il * (kB3 + 1) + seg);
 #pragma unroll
-            for (int m = 0; m < kZ3; ++m) v[m * kB3 * (kB3 + 1)] += SB[m];
+            for (int m = 0; m < kZ3; ++m) v[m * kB3 * (kB3 + 1)] += m & 1 ? SB[m / 2].y : SB[m / 2].x;
         }
         __syncthreads();
 #pragma unroll
