@@ -22,19 +22,21 @@
 // the clinical isocentre), so they fall into two z-cells (a third or more where the rows are
 // coarser, decided per chunk): the thread interpolates the levels L_j they share once along b,
 // and a row at x cells above the lowest one is L_0 + sum_j sat(x - j) (L_{j+1} - L_j) — six
-// shared loads and about 45 instructions for four samples, against sixteen loads and 90 for
-// four separate bilinear samples. L_0 is summed once for the four rows. Where a result is not
+// shared loads and about 40 instructions for four samples, against sixteen loads and 90 for
+// four separate bilinear samples. The planes of a chunk are unrolled for two, for three and for
+// any number of cells: a test and a loop in every plane cost 8 % (clinical 7.87 -> 7.23 ms). L_0 is summed once for the four rows. Where a result is not
 // finite (a NaN or infinite voxel in a level that only some of the rows use) every ray is
 // summed again from its own samples. Sums run per chunk and then over chunks, which keeps the
 // rounding of a ray well below one long sum's: error against 64 bits 1.5e-7 at the clinical size
-// (7.4e-7 with one running sum). Bounded by instruction issue (79 % of issue slots). Forward
-// projection by CUDA events, two rays per thread -> four: clinical 14.9 -> 7.8 ms, 2 x 128^3 /
-// 200 angles 2.07 -> 1.09 ms, 181 x 167 x 93 / 150 angles 2.10 -> 0.98 ms, 64^3 / 64 angles 48 -> 33 us.
+// (7.4e-7 with one running sum). Bounded by instruction issue (78 % of issue slots). Forward
+// projection by CUDA events, two rays per thread -> four: clinical 14.9 -> 7.23 ms, 2 x 128^3 /
+// 200 angles 2.07 -> 1.01 ms, 181 x 167 x 93 / 150 angles 2.10 -> 0.90 ms, 64^3 / 64 angles 48 -> 31 us.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
 #include <cmath>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "geom_impl.h"
@@ -317,9 +319,7 @@ __global__ void __launch_bounds__(kThreads, forward_ctas(BW, ZH, kP))
                     float low = 0.f;
                     float2 part[2];
                     part[0] = part[1] = make_float2(0.f, 0.f);
-                    // (planes past the volume are zero in the box)
-#pragma unroll
-                    for (int p = 0; p < kP; ++p) {
+                    auto plane = [&](int p, auto known) {  // known: cells, or 0
                         const float di = d0 + (float)p;
                         const float qb = fma_rn(di, c.dqb, c.qcb);
                         const float fb0 = floorf(qb), fb = qb - fb0;
@@ -333,26 +333,36 @@ __global__ void __launch_bounds__(kThreads, forward_ctas(BW, ZH, kP))
                         const float2 l01 = __ffma2_rn(make_float2(fb, fb), __ffma2_rn(va, make_float2(-1.f, -1.f), vb), va);
                         const float l2 = fmaf(fb, r[2 * BW + 1] - r[2 * BW], r[2 * BW]);
                         const float j1 = jz + 1.f, e1 = l01.y - l01.x, e2 = l2 - l01.y;
-                        const float2 e11 = make_float2(e1, e1);
+                        const float2 e11 = make_float2(e1, e1), e22 = make_float2(e2, e2);
                         low += l01.x;
                         part[0] = __ffma2_rn(make_float2(__saturatef(q0.x - jz), __saturatef(q0.y - jz)), e11, part[0]);
                         part[1] = __ffma2_rn(make_float2(__saturatef(q1.x - jz), __saturatef(q1.y - jz)), e11, part[1]);
                         part[0].y = fmaf(__saturatef(q0.y - j1), e2, part[0].y);
-                        part[1].x = fmaf(__saturatef(q1.x - j1), e2, part[1].x);
-                        part[1].y = fmaf(__saturatef(q1.y - j1), e2, part[1].y);
-                            if (cells > 2) {
-                                float l = l2;
+                        part[1] = __ffma2_rn(make_float2(__saturatef(q1.x - j1), __saturatef(q1.y - j1)), e22, part[1]);
+                        float l = l2;
+                        auto more = [&](int m) {
+                            const float *rm = r + (m + 1) * BW;
+                            const float ln = fmaf(fb, rm[1] - rm[0], rm[0]), e = ln - l, jm = jz + (float)m;
+                            part[0].y = fmaf(__saturatef(q0.y - jm), e, part[0].y);
+                            const float2 e2m = make_float2(e, e);
+                            part[1] = __ffma2_rn(make_float2(__saturatef(q1.x - jm), __saturatef(q1.y - jm)), e2m, part[1]);
+                            l = ln;
+                        };
+                        if constexpr (known.value == 3) {
+                            more(2);
+                        } else if constexpr (known.value == 0) {
 #pragma unroll 1
-                                for (int m = 2; m < cells; ++m) {
-                                    const float *rm = r + (m + 1) * BW;
-                                    const float ln = fmaf(fb, rm[1] - rm[0], rm[0]), e = ln - l, jm = jz + (float)m;
-                                    part[0].y = fmaf(__saturatef(q0.y - jm), e, part[0].y);
-                                    part[1].x = fmaf(__saturatef(q1.x - jm), e, part[1].x);
-                                    part[1].y = fmaf(__saturatef(q1.y - jm), e, part[1].y);
-                                    l = ln;
-                                }
-                            }
-                    }
+                            for (int m = 2; m < cells; ++m) more(m);
+                        }
+                    };
+                    // (planes past the volume are zero in the box)
+                    auto planes = [&](auto known) {
+#pragma unroll
+                        for (int p = 0; p < kP; ++p) plane(p, known);
+                    };
+                    if (cells == 2) planes(std::integral_constant<int, 2>());
+                    else if (cells == 3) planes(std::integral_constant<int, 3>());
+                    else planes(std::integral_constant<int, 0>());
                     acc[0] = __fadd2_rn(acc[0], __fadd2_rn(part[0], make_float2(low, low)));
                     acc[1] = __fadd2_rn(acc[1], __fadd2_rn(part[1], make_float2(low, low)));
                 } else if (mine && ci.flag != 0) {
