@@ -11,8 +11,8 @@
 // outside the image) as one box into a ring of stages; since a K-major core matrix
 // is 8 pixels x 16 B contiguous, every column tap is the same row region addressed
 // 16 B per pixel later, so each input row is read once per tile rather than once
-// per tap. One thread issues 128 x N x 16 tcgen05.mma, N = RPT x NPAD (the RPT
-// output rows' weights stacked), into several TMEM accumulators; sixteen epilogue
+// per tap. One warp issues 128 x N x 16 tcgen05.mma (its elected lane), N = RPT x NPAD
+// (the RPT output rows' weights stacked), into several TMEM accumulators; sixteen epilogue
 // warps drain them with tcgen05.ld. The packed weights (B) stay in shared memory
 // for the CTA's lifetime. The epilogue applies bias + LeakyReLU (BF16 row-blocked
 // out), a residual update of an FP32 channel-first state, or an activation mask.

@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(kThreads3, 3)
                             const float *src = raw + c + (h - 1) * kBC;
                             float2 *dst = E + c + (h - 1) * kEP;
                             rr = 1.f;
-#pragma unroll 4
+#pragma unroll 8
                             for (int r = 0; r < h; ++r) {
                                 const float p = src[-r * kBC];
                                 s0 -= p;
@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(kThreads3, 3)
                             float2 *dst = E + c + h * kEP;
                             rr = 0.f;
                             dst[0] = make_float2(0.f, 0.f);
-#pragma unroll 4
+#pragma unroll 8
                             for (int r = 0; r < nr - h; ++r) {
                                 const float p = src[r * kBC];
                                 s0 += p;
