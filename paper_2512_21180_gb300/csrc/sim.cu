@@ -153,8 +153,9 @@ __global__ void k_water_bone(const float *__restrict__ mu, long long nvox, long 
 // A thread takes one pixel in `group` frames (views of all items), so the air reading is summed
 // once. With FP64 draws the kernel was bound by the FP64 pipe (83 % of it); the draws of
 // poisson.cuh decide all but 1e-4 of them in FP32. 9.8 M pixels x 10 bins (CUDA events): 66.7 ms ->
-// 2.4 ms (41 G draws/s).
-__global__ void __launch_bounds__(256) k_poly_reading(const float *__restrict__ L, long long frames_per_item,
+// 2.19 ms (45 G draws/s). Bound by latency and issue (the samplers diverge: 17 of 32 lanes), so four
+// CTAs per SM of 64 registers beat three of 78 (2.37 ms) and five (2.21).
+__global__ void __launch_bounds__(256, 4) k_poly_reading(const float *__restrict__ L, long long frames_per_item,
                                                       long long nframes, int npix, long long group, const float *__restrict__ I0, PolyTab t,
                                                       unsigned long long seed, int noise, float *__restrict__ reading,
                                                       float *__restrict__ y, int32_t *__restrict__ counts) {
