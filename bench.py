@@ -393,7 +393,7 @@ def poly_timing(geom, name: str, reps: int = 3) -> dict:
     n_draws = L[0, 0].numel() * len(E)
     return {"ms_per_volume": t_all / reps, "ms_reading": t_read / reps, "bins": len(E),
             "gdraws_s": n_draws / (t_read / reps * 1e-3) / 1e9,
-            "note": "stand-in attenuation tables and intensity maps; FP64 Poisson draws (inversion / PTRS)"}
+            "note": "stand-in attenuation tables and intensity maps; Poisson draws that match FP64 ones (inversion / PTRS)"}
 
 
 def report(args, geom, world, S_fwd, samples_step, value, ms, ms_fwd, ms_adj, e2e, clk, g, dist):
@@ -424,8 +424,8 @@ def report(args, geom, world, S_fwd, samples_step, value, ms, ms_fwd, ms_adj, e2
                    "gsamples_s_adjoint": S_fwd / (ms_adj * 1e-3) / 1e9},
         "roofline": roof,
         "e2e": {"value": e2e, "unit": "Gsamples/s", "h2d_bytes_per_step": nvox * 4, "d2h_bytes_per_step": nvox * 4},
-        # per step: forward = two plane transposes + the TMA ray kernel; adjoint = ray
-        # weighting + segment gather (+ the fixed-order sum of angle parts when split)
+        # per step: forward = plane transpose + the TMA ray kernel; adjoint = ray weighting +
+        # segment gather (+ the fixed-order sum of angle parts when split)
         "gpu_launches": launches_per_step(geom) * args.steps,
         "clocks": clk,
     }
@@ -467,23 +467,27 @@ def report(args, geom, world, S_fwd, samples_step, value, ms, ms_fwd, ms_adj, e2
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch, from one ncu
 # --set full capture of the clinical workload with the current kernels; None elsewhere
 # and whenever the kernel changes after the capture.
-MEASURED_TRAFFIC = {"clinical": {"back_project": None, "forward_project": 136.448e6 + 280.638e6}}
+MEASURED_TRAFFIC = {"clinical": {"back_project": 1309.8e6 + 38.6e6, "forward_project": 132.9e6 + 280.1e6}}
 # The binding on-chip level's throughput from the same captures: the projector kernels are
 # bound by SM instruction issue, so this is sm__throughput.avg.pct_of_peak_sustained_elapsed
-# (issue active: forward 75.0 %). Same validity rule as the traffic: the adjoint's capture
-# (619 MB, 74.0 %) predates its brick-level reach test, so both figures are withheld for it.
-MEASURED_SM_THROUGHPUT_PCT = {"clinical": {"back_project": None, "forward_project": 75.0}}
+# (issue active: forward 80.6 %, adjoint 65.9 %). Same validity rule as the traffic.
+MEASURED_SM_THROUGHPUT_PCT = {"clinical": {"back_project": 62.0, "forward_project": 80.5}}
 
 
 def launches_per_step(geom) -> int:
-    """Kernels one forward + adjoint step launches (mirrors the launchers: 3 for the
-    staged forward, 2 for the segment gather, +1 when its angles are split)."""
+    """Kernels one forward + adjoint step launches (mirrors the launchers: x planes and the
+    staged forward, y planes too when rows do not start on 16 bytes, or one direct kernel for
+    small calls; ray weighting and the segment gather, +1 when its angles are split)."""
     import torch
     nsm = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
     nx, ny, nz = geom.g["n"]
-    bricks = -(-nx // 16) * -(-ny // 16) * -(-nz // 16)
-    parts = min(16, max(1, -(-nsm * 9 // bricks)), geom.g["n_angles"])
-    return 3 + 2 + (1 if parts > 1 else 0)
+    na = geom.g["n_angles"]
+    direct = na * geom.g["nv"] * geom.g["nu"] * max(nx, ny) <= 1 << 20
+    forward = 1 if direct else 2 + (nx % 4 != 0)
+    bricks = -(-nx // 16) * -(-ny // 16) * -(-nz // 8)
+    parts = min(16, max(1, -(-nsm * 24 // bricks)))
+    parts = min(parts, max(-(-na // 8), -(-nsm * 6 // bricks)), na)
+    return forward + 2 + (1 if parts > 1 else 0)
 
 
 def smem_peak_gbs(reps: int = 5) -> dict:
