@@ -544,6 +544,16 @@ int cbct_smem_probe(int ctas_per_sm, int iters, float *sink, long long *bytes, v
  * range. */
 int cbct_wait_probe(const cbct_geom *g, long long limit_ns, int *waited_ok, void *stream);
 
+/* Test of the vote by which a CTA leaves its tile loop together after a wait that gave up
+ * (no counterpart in the paper). One CTA of 96 threads runs three tiles of that loop on a
+ * barrier: each thread waits at most limit_ns nanoseconds (1 .. 1e7; threads `late` and above ten times
+ * that), the CTA votes, and a tile is taken as odd when thread `odd` (negative: none) reports odd data
+ * in the second one. arrive: 0 nothing completes the barrier, 1 it completes at once, 2 after three
+ * times the limit, so that only the patient threads see it. out (device): 96 counts of tiles taken
+ * normally, then 96 of tiles taken as odd, written only when no thread gave up. Asynchronous on
+ * `stream`. Errors: CBCT_EINVAL for NULL pointers or a limit out of range. */
+int cbct_vote_probe(const cbct_geom *g, long long limit_ns, int late, int arrive, int odd, int *out, void *stream);
+
 /* Read (and with clear = 1 reset) the model's device status word: 0 = ok, 1 = one of
  * its convolution kernels (forward, input-gradient or weight-gradient) gave up waiting
  * on its tensor-core pipeline (it then left its outputs unwritten, or wrote a zero

@@ -92,6 +92,7 @@ SIGNATURES = {
     "lpd_get_grads": (I32, [P, P, I64]),
     "cbct_masked_mse": (I32, [P, P, P, F32, I64, P, P, P]),
     "cbct_wait_probe": (I32, [P, I64, P, P]),
+    "cbct_vote_probe": (I32, [P, I64, I32, I32, I32, P, P]),
     "lpd_get_perms": (I32, [P, P]),
     "cbct_smem_probe": (I32, [I32, I32, P, ctypes.POINTER(I64), P]),
     "lpd_set_perms": (I32, [P, P]),

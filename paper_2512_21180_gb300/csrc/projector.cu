@@ -477,8 +477,8 @@ __global__ void __launch_bounds__(kThreads3, 3)
                 }
                 // a wait that gave up ends the sweep for every thread; a tile whose sums are not
                 // finite takes its rows one by one
-                const int flags = __syncthreads_or((ok ? 0 : 2) | (odd ? 1 : 0));
-                if (flags & 2) {
+                const CtaVote vote = cta_vote(!ok, odd);
+                if (vote.gave_up) {
                     ok = false;
                     break;
                 }
@@ -518,7 +518,7 @@ __global__ void __launch_bounds__(kThreads3, 3)
                         const float step = t * drz, irs = __fdividef(1.0f, step);
                         // z of the tile's middle row relative to z0 - 1
                         const float qh = fmaf(t, rzh, Szb);
-                        if (!(flags & 1)) {
+                        if (!vote.odd) {
                             // x(m): tile row coordinate of z0 - 1 + m, plus one; the first row above
                             // is floor(x). In units of step, the rows of interval m weigh
                             // S1 = T - (x - 1 - h) S0 on the upper voxel and irs S0 - S1 on the lower.

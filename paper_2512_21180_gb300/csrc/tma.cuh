@@ -73,6 +73,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, int *s
     }
 }
 
+// What a CTA's threads found: whether one gave up a wait, and whether one saw something odd in
+// its data. Every thread gets the same answer. (A barrier's OR is a vote, not the OR of bits: two
+// questions take two votes, the second only where the first found anything.)
+struct CtaVote {
+    bool gave_up, odd;
+};
+__device__ __forceinline__ CtaVote cta_vote(bool gave_up, bool odd) {
+    if (!__syncthreads_or(gave_up || odd)) return CtaVote{false, false};
+    const bool g = __syncthreads_or(gave_up) != 0;
+    return CtaVote{g, __syncthreads_or(odd) != 0};
+}
+
 // 3D tiled TMA load of a box into shared memory, completion counted on `bar`.
 __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, int c0, int c1, int c2, uint64_t *bar) {
     asm volatile(

@@ -31,6 +31,44 @@ __global__ void k_wait_probe(int *status, uint64_t limit_ns, int *waited_ok) {
     __syncthreads();
 }
 
+// A CTA of 96 threads that runs the staged kernels' tile loop: every thread waits for the tile,
+// the CTA votes, and a wait that gave up ends the loop for all of it before anything is
+// written. late: threads from `late` on take ten times the limit, so that the others
+// give up first; arrive: 0 the barrier never completes, 1 it completes at once, 2 thread 95
+// completes it after three times the limit (the patient threads succeed, the others gave up). odd: the
+// thread that reports odd data in the second tile (negative: none). out[thread] counts tiles taken
+// normally, out[96 + thread] tiles taken as odd.
+__global__ void k_vote_probe(int *status, uint64_t limit_ns, int late, int arrive, int odd, int *out) {
+    __shared__ __align__(8) uint64_t bar;
+    if (threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    int normal = 0, odds = 0;
+    bool ok = true;
+    for (int tile = 0; tile < 3; ++tile) {
+        if (threadIdx.x == 0 && arrive == 1) mbar_arrive(&bar);
+        if (threadIdx.x == 95 && arrive == 2) {
+            const uint64_t t0 = global_ns();
+            while (global_ns() - t0 < 3 * limit_ns) {}
+            mbar_arrive(&bar);
+        }
+        ok = mbar_wait(&bar, (uint32_t)(tile & 1), status, (int)threadIdx.x >= late ? 10 * limit_ns : limit_ns);
+        const CtaVote v = cta_vote(!ok, ok && (int)threadIdx.x == odd && tile == 1);
+        if (v.gave_up) {
+            ok = false;
+            break;
+        }
+        if (v.odd) ++odds;
+        else ++normal;
+        __syncthreads();
+    }
+    if (!ok) return;
+    out[threadIdx.x] = normal;
+    out[96 + threadIdx.x] = odds;
+}
+
 }  // namespace
 }  // namespace cbct
 
@@ -41,5 +79,13 @@ extern "C" int cbct_wait_probe(const cbct_geom *g, long long limit_ns, int *wait
         return fail(CBCT_EINVAL, "cbct_wait_probe: need a geometry, a device counter and 1 <= limit_ns <= 1e8");
     k_wait_probe<<<1, 64, 0, (cudaStream_t)stream>>>(g->status, (uint64_t)limit_ns, waited_ok);
     CBCT_LAUNCH_CHECK("cbct_wait_probe");
+    return 0;
+}
+
+extern "C" int cbct_vote_probe(const cbct_geom *g, long long limit_ns, int late, int arrive, int odd, int *out, void *stream) {
+    if (!g || !out || limit_ns < 1 || limit_ns > 10000000LL)
+        return fail(CBCT_EINVAL, "cbct_vote_probe: need a geometry, a device array and 1 <= limit_ns <= 1e7");
+    k_vote_probe<<<1, 96, 0, (cudaStream_t)stream>>>(g->status, (uint64_t)limit_ns, late, arrive, odd, out);
+    CBCT_LAUNCH_CHECK("cbct_vote_probe");
     return 0;
 }
