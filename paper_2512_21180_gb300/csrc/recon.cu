@@ -268,7 +268,8 @@ __global__ void __launch_bounds__(N / 8, N <= 1024 ? 8 : N == 2048 ? 4 : 2)
         }
         // (also: the previous pair's last reads are done) a row with a non-finite value stays out of
         // the transform, which would spread it over both rows
-        const int bad = __syncthreads_or((ok0 ? 0 : 1) | (ok1 ? 0 : 2));
+        int bad = __syncthreads_or(!ok0 || !ok1);  // (a vote: which of the rows takes a second one)
+        if (bad) bad = (__syncthreads_or(!ok0) ? 1 : 0) | (__syncthreads_or(!ok1) ? 2 : 0);
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
             if (bad & 1) v[m].x = 0.f;

@@ -62,3 +62,37 @@ def test_non_finite_row_stays_in_its_row(O, name, value):
     assert int(near.sum()) > 100
     if value != 3e38:
         assert int((~torch.isfinite(got[near])).sum()) > 50
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), 3e38])
+@pytest.mark.parametrize("rows", [(12,), (13,), (12, 13)])
+def test_a_bad_row_leaves_its_partner_alone(O, rows, value):
+    """Rows 12 and 13 share a transform: one of them with four bad pixels, or both. Every voxel whose
+    detector row lies a row away from the bad ones keeps its bits, the partner's own band included."""
+    g = CASES["fft1024"]
+    geom = P.Geometry(g)
+    y = to_gpu(I.random_volume((1,) + geom.proj_shape, 6))
+    k = 5
+    # the other angles, and the bad rows, contribute nothing: what is left is the partner's band
+    y[0, :k] = 0.0
+    y[0, k + 1:] = 0.0
+    for iv in rows:
+        y[0, k, iv] = 0.0
+    clean = ops.fdk(geom, y)
+    for iv in rows:
+        y[0, k, iv, 40:44] = value
+    got = ops.fdk(geom, y)
+    z, yy, x = (torch.arange(n, device="cuda", dtype=torch.float64) - 0.5 * (n - 1) for n in geom.vol_shape)
+    th = 2 * np.pi * k / g["n_angles"]
+    U = 1000.0 - 4.0 * (x[None, :] * np.cos(th) + yy[:, None] * np.sin(th))
+    fv = ((1536.0 / U)[None] * (4.0 * z)[:, None, None] / g["dv"] + 0.5 * (g["nv"] - 1))[None]
+    far = ((fv < min(rows) - 1.01) | (fv > max(rows) + 1.01))
+    assert int(far.sum()) > 1000
+    if value == 3e38:   # finite, but the transform overflows: the partner is summed tap by tap
+        assert float((got[far] - clean[far]).abs().max()) <= 1e-6 * float(clean.abs().max())
+    else:
+        assert torch.equal(got[far], clean[far])
+        near = torch.zeros_like(far)
+        for iv in rows:
+            near |= (fv - iv).abs() < 0.9
+        assert int((~torch.isfinite(got[near])).sum()) > 50
