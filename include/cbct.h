@@ -545,12 +545,14 @@ int cbct_smem_probe(int ctas_per_sm, int iters, float *sink, long long *bytes, v
 int cbct_wait_probe(const cbct_geom *g, long long limit_ns, int *waited_ok, void *stream);
 
 /* Test of the vote by which a CTA leaves its tile loop together after a wait that gave up
- * (no counterpart in the paper). One CTA of 96 threads runs three tiles of that loop on a
- * barrier: each thread waits at most limit_ns nanoseconds (1 .. 1e7; threads `late` and above ten times
+ * (no counterpart in the paper). Three waiting warps run three tiles of that loop on a
+ * barrier that a fourth completes: each thread waits at most limit_ns nanoseconds (1 .. 1e7; threads `late` and above ten times
  * that), the CTA votes, and a tile is taken as odd when thread `odd` (negative: none) reports odd data
  * in the second one. arrive: 0 nothing completes the barrier, 1 it completes at once, 2 after three
  * times the limit, so that only the patient threads see it. out (device): 96 counts of tiles taken
- * normally, then 96 of tiles taken as odd, written only when no thread gave up. Asynchronous on
+ * normally, then 96 of tiles taken as odd, written only when no thread gave up; then 96 counts of a
+ * loop of three such waits in which every lane stays with its warp: 100 times the steps that the thread's
+ * waits completed, plus 96 (the lanes that took part in its warp's sums), always written. Asynchronous on
  * `stream`. Errors: CBCT_EINVAL for NULL pointers or a limit out of range. */
 int cbct_vote_probe(const cbct_geom *g, long long limit_ns, int late, int arrive, int odd, int *out, void *stream);
 

@@ -292,7 +292,6 @@ __global__ void __launch_bounds__(kWsThreads) k_conv_tc(const __grid_constant__ 
     uint64_t *acce = accf + kMaxAcc;
     float *sbias = reinterpret_cast<float *>(acce + kMaxAcc);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sbias + NPAD);
-    int *abort_flag = reinterpret_cast<int *>(tmem_slot + 1);
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     constexpr int kAcc = conv_nacc(kN);
@@ -313,7 +312,6 @@ __global__ void __launch_bounds__(kWsThreads) k_conv_tc(const __grid_constant__ 
             mbar_init(&accf[j], 1);
             mbar_init(&acce[j], 4);
         }
-        *abort_flag = 0;
         fence_mbar_init();
     }
     if (tid < NPAD) sbias[tid] = (a.bias && tid < a.cout) ? a.bias[tid] : 0.f;
@@ -351,10 +349,7 @@ __global__ void __launch_bounds__(kWsThreads) k_conv_tc(const __grid_constant__ 
             int c = 0, s = 0;
             uint32_t ph = 0;
             for (long long i = 0; i < total; ++i) {
-                if (i >= nst && !mbar_wait(&empty[s], ph ^ 1u, a.status)) {
-                    *abort_flag = 1;
-                    break;
-                }
+                if (i >= nst && !mbar_wait(&empty[s], ph ^ 1u, a.status)) break;
                 const int d2 = tc.d + (nch == 3 ? c - 1 : 0);
                 if (d2 < 0 || d2 >= a.D) {
                     mbar_arrive_expect_tx(&full[s], 0u);  // plane outside the volume: no MMAs either
@@ -384,22 +379,18 @@ __global__ void __launch_bounds__(kWsThreads) k_conv_tc(const __grid_constant__ 
             TileCoord tc = tile_coord(t_begin, a.D, nh, ntw);
             int s = 0;
             uint32_t ph = 0;
-            for (long long j = 0; j < my_tiles && !*abort_flag; ++j) {
+            bool alive = true;
+            for (long long j = 0; j < my_tiles; ++j) {
                 const int ab = (int)(j % kAcc);
-                if (j >= kAcc && !mbar_wait(&acce[ab], (uint32_t)(((j / kAcc) - 1) & 1), a.status)) {
-                    *abort_flag = 1;
-                    break;
-                }
-                __syncwarp();
+                if (j >= kAcc && !mbar_wait_warp(&acce[ab], (uint32_t)(((j / kAcc) - 1) & 1), a.status)) break;
                 tc_fence_after();
                 const uint32_t dt = tmem + (uint32_t)(ab * kN);
                 uint32_t acc_flag = 0;  // the tile's first MMA overwrites the accumulator
                 for (int c = 0; c < nch; ++c) {
-                    if (!mbar_wait(&full[s], ph, a.status)) {
-                        *abort_flag = 1;
+                    if (!mbar_wait_warp(&full[s], ph, a.status)) {
+                        alive = false;
                         break;
                     }
-                    __syncwarp();
                     const int d2 = tc.d + (nch == 3 ? c - 1 : 0);
                     if (d2 >= 0 && d2 < a.D) {
                         tc_fence_after();
@@ -445,7 +436,7 @@ __global__ void __launch_bounds__(kWsThreads) k_conv_tc(const __grid_constant__ 
                         ph ^= 1u;
                     }
                 }
-                if (*abort_flag) break;
+                if (!alive) break;
                 mma_commit(&accf[ab], leader);
                 tile_next(tc, a.D, nh, a.W);
             }
@@ -458,14 +449,13 @@ __global__ void __launch_bounds__(kWsThreads) k_conv_tc(const __grid_constant__ 
 #pragma unroll
         for (int c = 0; c < NPAD; ++c) bias[c] = sbias[c];
         TileCoord tc = tile_coord(t_begin + q, a.D, nh, ntw);
+        bool alive = true;
         for (long long j = q; j < my_tiles; j += kEpiGroups) {
             const int ab = (int)(j % kAcc);
-            if (!mbar_wait(&accf[ab], (uint32_t)((j / kAcc) & 1), a.status)) {
-                *abort_flag = 1;
-                break;
-            }
+            mbar_wait_alive(alive, &accf[ab], (uint32_t)((j / kAcc) & 1), a.status);
             tc_fence_after();
-            const int w = tc.w0 + wq * 32 + lane;
+            // (a lane whose wait gave up takes a pixel past the image: nothing is stored)
+            const int w = alive ? tc.w0 + wq * 32 + lane : a.W;
             // one output row at a time (NPAD accumulator columns each); the accumulator is
             // released after the last row's columns are in registers
 #pragma unroll
@@ -478,7 +468,7 @@ __global__ void __launch_bounds__(kWsThreads) k_conv_tc(const __grid_constant__ 
                 if (o == RPT - 1) {
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(&acce[ab]);
+                    if (lane == 0 && alive) mbar_arrive(&acce[ab]);
                 }
                 const int h = tc.th * RPT + o;
                 float acc[NPAD];
@@ -627,8 +617,7 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
     uint64_t *empty = full + kWgStages;
     uint64_t *done = empty + kWgStages, *drained = done + 1;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drained + 1);
-    int *abort_flag = reinterpret_cast<int *>(tmem_slot + 1);
-    int *used = abort_flag + 1;  // [3]: accumulator dw received an MMA in this segment
+    int *used = reinterpret_cast<int *>(tmem_slot + 1);  // [3]: accumulator dw received an MMA in this segment
     float *xch = reinterpret_cast<float *>(used + 3);  // [3][16][32]: tap sums on their way between warps
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int ndd = a.taps3d ? 3 : 1, gpd = (int)gridDim.x / ndd;
@@ -645,7 +634,6 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
         }
         mbar_init(done, 2);     // a segment's MMAs: their commit + the MMA thread's release of used[]
         mbar_init(drained, 4);  // its accumulators read by the four epilogue warps
-        *abort_flag = 0;
         for (int i = 0; i < 3; ++i) used[i] = 0;
         fence_mbar_init();
     }
@@ -690,10 +678,7 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
             int s = 0;
             uint32_t ph = 0;
             for (long long i = 0; i < my_tiles; ++i) {
-                if (i >= kWgStages && !mbar_wait(&empty[s], ph ^ 1u, a.status)) {
-                    *abort_flag = 1;
-                    break;
-                }
+                if (i >= kWgStages && !mbar_wait(&empty[s], ph ^ 1u, a.status)) break;
                 const int d2 = tc.d + (a.taps3d ? dd - 1 : 0);
                 if (d2 < 0 || d2 >= a.D) {
                     mbar_arrive_expect_tx(&full[s], 0u);  // input plane outside the volume: no MMAs
@@ -728,6 +713,7 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
             uint32_t ph = 0;
             uint32_t usedm = 0;  // bit dw: accumulator initialised
             int seg = 0;
+            bool alive = true;
             // the segment's accumulators to the epilogue (a segment without MMAs, in a CTA without
             // tiles, arrives directly instead of committing)
             auto hand_over = [&]() {
@@ -740,21 +726,16 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
                 usedm = 0;
                 ++seg;
             };
-            for (long long i = 0; i < my_tiles && !*abort_flag; ++i) {
-                while (i == seg_end(seg)) {
+            for (long long i = 0; i < my_tiles && alive; ++i) {
+                while (alive && i == seg_end(seg)) {
                     hand_over();
-                    if (!mbar_wait(drained, (uint32_t)((seg - 1) & 1), a.status)) {
-                        *abort_flag = 1;
-                        break;
-                    }
-                    __syncwarp();
+                    alive = mbar_wait_warp(drained, (uint32_t)((seg - 1) & 1), a.status);
                     tc_fence_after();
                 }
-                if (*abort_flag || !mbar_wait(&full[s], ph, a.status)) {
-                    *abort_flag = 1;
+                if (!alive || !mbar_wait_warp(&full[s], ph, a.status)) {
+                    alive = false;
                     break;
                 }
-                __syncwarp();
                 const int d2 = tc.d + (a.taps3d ? dd - 1 : 0);
                 if (d2 >= 0 && d2 < a.D) {
                     tc_fence_after();
@@ -780,10 +761,11 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
                     ph ^= 1u;
                 }
             }
-            hand_over();
-            for (; seg < nseg;) {  // (segments past the tiles of a CTA with few)
-                if (!mbar_wait(drained, (uint32_t)((seg - 1) & 1), a.status)) break;
-                hand_over();
+            // (after a wait that gave up nothing more is handed over: the epilogue's own waits run out)
+            if (alive) hand_over();
+            while (alive && seg < nseg) {  // (segments past the tiles of a CTA with few)
+                alive = mbar_wait_warp(drained, (uint32_t)((seg - 1) & 1), a.status);
+                if (alive) hand_over();
             }
         }
     } else {
@@ -791,14 +773,12 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
         int s = 0;
         uint32_t ph = 0;
         long long i = 0;
+        bool alive = true;
         for (int seg = 0; seg < nseg; ++seg) {
             for (; bias && i < seg_end(seg); ++i) {
                 // the lane's pixels of both dY rows (zero outside the image)
-                if (!mbar_wait(&full[s], ph, a.status)) {
-                    *abort_flag = 1;
-                    break;
-                }
-                if (warp < cgo) {
+                mbar_wait_alive(alive, &full[s], ph, a.status);
+                if (alive && warp < cgo) {
                     const uint4 *src = reinterpret_cast<const uint4 *>(sm + s * kStage + kWgXBytes + warp * 2048) + lane;
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
@@ -813,7 +793,7 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
                     }
                 }
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&empty[s]);
+                if (lane == 0 && alive) mbar_arrive(&empty[s]);
                 if (++s == kWgStages) {
                     s = 0;
                     ph ^= 1u;
@@ -822,12 +802,12 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
             // warp w holds accumulator rows 32 w .. 32 w + 31 = input row r = w, input channel = lane;
             // columns (o, co). Pair (r, o) is tap dh = r - 1 - o: row r's o = 1 columns go through
             // shared memory to row r - 1's o = 0 ones, 16 columns at a time
-            const bool ok = mbar_wait(done, (uint32_t)(seg & 1), a.status) && !*abort_flag;
+            mbar_wait_alive(alive, done, (uint32_t)(seg & 1), a.status);
             tc_fence_after();
             float *pb = partial + (((long long)dd * gpd + cta) * nseg + seg) * a.cout * 9 * a.cin;
 #pragma unroll 1
             for (int dw = 0; dw < 3; ++dw) {
-                const bool valid = ok && used[dw];
+                const bool valid = alive && used[dw];
 #pragma unroll 1
                 for (int c0 = 0; c0 < NCG * 8; c0 += 16) {
                     float v[16];
@@ -853,7 +833,7 @@ __global__ void __launch_bounds__(kWgThreads) k_conv_wgrad_tc(const __grid_const
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(drained);
+            if (lane == 0 && alive) mbar_arrive(drained);
         }
         if (bias) {
 #pragma unroll

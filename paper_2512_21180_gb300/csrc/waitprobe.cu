@@ -31,30 +31,51 @@ __global__ void k_wait_probe(int *status, uint64_t limit_ns, int *waited_ok) {
     __syncthreads();
 }
 
-// A CTA of 96 threads that runs the staged kernels' tile loop: every thread waits for the tile,
-// the CTA votes, and a wait that gave up ends the loop for all of it before anything is
-// written. late: threads from `late` on take ten times the limit, so that the others
-// give up first; arrive: 0 the barrier never completes, 1 it completes at once, 2 thread 95
-// completes it after three times the limit (the patient threads succeed, the others gave up). odd: the
+// Three waiting warps, and a fourth that completes the barriers, run the staged kernels' tile loop:
+// every thread of the three waits for the tile, the CTA votes, and a wait that gave up ends
+// the loop for all of it before anything is written. late: threads from `late` on take ten times the limit, so that the others
+// give up first; arrive: 0 the barrier never completes, 1 it completes at once, 2 it
+// completes after three times the limit (the patient threads succeed, the others gave up). odd: the
 // thread that reports odd data in the second tile (negative: none). out[thread] counts tiles taken
-// normally, out[96 + thread] tiles taken as odd.
+// normally, out[96 + thread] tiles taken as odd. Before that each warp runs three steps of the
+// convolutions' loops on another barrier, a warp-wide sum in each step: out[192 + thread] is
+// 100 (steps that the thread saw alive) + lanes counted by the sums of all steps.
 __global__ void k_vote_probe(int *status, uint64_t limit_ns, int late, int arrive, int odd, int *out) {
-    __shared__ __align__(8) uint64_t bar;
+    __shared__ __align__(8) uint64_t bar, wbar;
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
+        mbar_init(&wbar, 1);
         fence_mbar_init();
     }
     __syncthreads();
+    const uint64_t limit = (int)threadIdx.x >= late ? 10 * limit_ns : limit_ns;
+    const bool waits = threadIdx.x < 96;
+    auto complete = [&](uint64_t *b) {  // thread 96
+        if (threadIdx.x != 96 || arrive == 0) return;
+        const uint64_t t0 = global_ns();
+        while (arrive == 2 && global_ns() - t0 < 3 * limit_ns) {}
+        mbar_arrive(b);
+    };
+    int steps = 0, lanes = 0;
+    bool alive = true;
+    for (int step = 0; step < 3; ++step) {
+        if (waits) {
+            mbar_wait_alive(alive, &wbar, (uint32_t)(step & 1), status, limit);
+            if (alive) ++steps;
+            int one = 1;
+            for (int o = 16; o > 0; o >>= 1) one += __shfl_xor_sync(0xffffffffu, one, o);
+            lanes += one;
+        } else {
+            complete(&wbar);
+        }
+        __syncthreads();
+    }
+    if (waits) out[192 + threadIdx.x] = 100 * steps + lanes;
     int normal = 0, odds = 0;
     bool ok = true;
     for (int tile = 0; tile < 3; ++tile) {
-        if (threadIdx.x == 0 && arrive == 1) mbar_arrive(&bar);
-        if (threadIdx.x == 95 && arrive == 2) {
-            const uint64_t t0 = global_ns();
-            while (global_ns() - t0 < 3 * limit_ns) {}
-            mbar_arrive(&bar);
-        }
-        ok = mbar_wait(&bar, (uint32_t)(tile & 1), status, (int)threadIdx.x >= late ? 10 * limit_ns : limit_ns);
+        if (waits) ok = mbar_wait(&bar, (uint32_t)(tile & 1), status, limit);
+        else complete(&bar);
         const CtaVote v = cta_vote(!ok, ok && (int)threadIdx.x == odd && tile == 1);
         if (v.gave_up) {
             ok = false;
@@ -64,7 +85,7 @@ __global__ void k_vote_probe(int *status, uint64_t limit_ns, int late, int arriv
         else ++normal;
         __syncthreads();
     }
-    if (!ok) return;
+    if (!ok || !waits) return;
     out[threadIdx.x] = normal;
     out[96 + threadIdx.x] = odds;
 }
@@ -85,7 +106,7 @@ extern "C" int cbct_wait_probe(const cbct_geom *g, long long limit_ns, int *wait
 extern "C" int cbct_vote_probe(const cbct_geom *g, long long limit_ns, int late, int arrive, int odd, int *out, void *stream) {
     if (!g || !out || limit_ns < 1 || limit_ns > 10000000LL)
         return fail(CBCT_EINVAL, "cbct_vote_probe: need a geometry, a device array and 1 <= limit_ns <= 1e7");
-    k_vote_probe<<<1, 96, 0, (cudaStream_t)stream>>>(g->status, (uint64_t)limit_ns, late, arrive, odd, out);
+    k_vote_probe<<<1, 128, 0, (cudaStream_t)stream>>>(g->status, (uint64_t)limit_ns, late, arrive, odd, out);
     CBCT_LAUNCH_CHECK("cbct_vote_probe");
     return 0;
 }

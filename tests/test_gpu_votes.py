@@ -1,5 +1,6 @@
 """How a pipelined kernel leaves when one of its waits gives up: all threads of the CTA together,
-with nothing written, whichever of them gave up; and a tile that one thread finds odd is odd for
+with nothing written, whichever of them gave up; a lane of a warp-wide loop stays with its
+warp to the end; and a tile that one thread finds odd is odd for
 all of them while the loop goes on. The waits expire on a barrier in shared memory after a short
 limit of the GPU's global timer (no fault, no hang)."""
 import pytest
@@ -21,11 +22,14 @@ def env():
 def run(env, late, arrive, odd):
     L, geom = env
     assert geom.device_status(clear=True) == 0
-    out = torch.full((192,), -7, dtype=torch.int32, device="cuda")
+    out = torch.full((288,), -7, dtype=torch.int32, device="cuda")
     L.check(L.load().cbct_vote_probe(geom.handle, 2_000_000, late, arrive, odd, out.data_ptr(),
                                      torch.cuda.current_stream().cuda_stream), "cbct_vote_probe")
     torch.cuda.synchronize()
-    return out, geom.device_status(clear=True)
+    # every lane took part in all its warp's sums; a lane whose wait gave up did nothing else
+    seen = [3 if arrive == 1 or (arrive == 2 and t >= late) else 0 for t in range(96)]
+    assert out[192:].tolist() == [100 * s + 96 for s in seen]
+    return out[:192], geom.device_status(clear=True)
 
 
 @pytest.mark.parametrize("late,arrive", [(96, 0), (0, 0), (40, 0), (1, 0), (95, 0), (40, 2), (64, 2), (95, 2)])
