@@ -546,13 +546,14 @@ int cbct_wait_probe(const cbct_geom *g, long long limit_ns, int *waited_ok, void
 
 /* Test of the vote by which a CTA leaves its tile loop together after a wait that gave up
  * (no counterpart in the paper). Three waiting warps run three tiles of that loop on a
- * barrier that a fourth completes: each thread waits at most limit_ns nanoseconds (1 .. 1e7; threads `late` and above ten times
- * that), the CTA votes, and a tile is taken as odd when thread `odd` (negative: none) reports odd data
+ * barrier that a fourth completes: each thread waits at most limit_ns nanoseconds (1 .. 1e7;
+ * threads `late` and above ten times that), the CTA votes, and a tile is taken as odd when thread `odd` (negative: none) reports odd data
  * in the second one. arrive: 0 nothing completes the barrier, 1 it completes at once, 2 after three
  * times the limit, so that only the patient threads see it. out (device): 96 counts of tiles taken
- * normally, then 96 of tiles taken as odd, written only when no thread gave up; then 96 counts of a
- * loop of three such waits in which every lane stays with its warp: 100 times the steps that the thread's
- * waits completed, plus 96 (the lanes that took part in its warp's sums), always written. Asynchronous on
+ * normally, then 96 of tiles taken as odd, written only when no thread gave up; then 96 counts, always
+ * written, of two loops of three such waits: 1000 times the steps that the thread passed in a loop that
+ * it leaves when a wait gives up, plus 100 times those of a loop in which it stays with its warp, plus 96
+ * (the lanes that took part in that warp's sums). Asynchronous on
  * `stream`. Errors: CBCT_EINVAL for NULL pointers or a limit out of range. */
 int cbct_vote_probe(const cbct_geom *g, long long limit_ns, int late, int arrive, int odd, int *out, void *stream);
 

@@ -302,7 +302,9 @@ __global__ void __launch_bounds__(kThreads, forward_ctas(BW, ZH, kP))
             for (int ch = 0; ch < nch; ++ch) {
                 const int q = gc + ch, s = q % kStages, use = q / kStages;
                 if (!mbar_wait(&full[s], use & 1, status)) {
+                    // (by vote or by staying, as in the convolutions, cost 3 % of the kernel)
                     abort_flag = 1;
+                    leave_warp_loop(nch - ch);
                     break;
                 }
                 const ChunkInfo ci = info[ch];

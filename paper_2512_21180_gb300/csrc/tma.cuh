@@ -90,6 +90,13 @@ __device__ __forceinline__ void mbar_wait_alive(bool &alive, uint64_t *bar, uint
     alive = mbar_wait(bar, parity, status, alive ? limit_ns : 0) && alive;
 }
 
+// By leaving, for a loop whose only warp-wide step is one __syncwarp() in each iteration: the lane that
+// leaves makes the barriers of its remaining iterations first (any call site counts).
+__device__ __forceinline__ void leave_warp_loop(int iterations) {
+#pragma unroll 1
+    for (; iterations > 0; --iterations) __syncwarp();
+}
+
 // What a CTA's threads found: whether one gave up a wait, and whether one saw something odd in
 // its data. Every thread gets the same answer. (A barrier's OR is a vote, not the OR of bits: two
 // questions take two votes, the second only where the first found anything.)

@@ -38,13 +38,15 @@ __global__ void k_wait_probe(int *status, uint64_t limit_ns, int *waited_ok) {
 // completes after three times the limit (the patient threads succeed, the others gave up). odd: the
 // thread that reports odd data in the second tile (negative: none). out[thread] counts tiles taken
 // normally, out[96 + thread] tiles taken as odd. Before that each warp runs three steps of the
-// convolutions' loops on another barrier, a warp-wide sum in each step: out[192 + thread] is
+// convolutions' loops on another barrier, a warp-wide sum in each step, and three of the forward
+// projector's on a third one, which a lane leaves: out[192 + thread] is 1000 (steps of the latter) +
 // 100 (steps that the thread saw alive) + lanes counted by the sums of all steps.
 __global__ void k_vote_probe(int *status, uint64_t limit_ns, int late, int arrive, int odd, int *out) {
-    __shared__ __align__(8) uint64_t bar, wbar;
+    __shared__ __align__(8) uint64_t bar, wbar, lbar;
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
         mbar_init(&wbar, 1);
+        mbar_init(&lbar, 1);
         fence_mbar_init();
     }
     __syncthreads();
@@ -70,7 +72,21 @@ __global__ void k_vote_probe(int *status, uint64_t limit_ns, int late, int arriv
         }
         __syncthreads();
     }
-    if (waits) out[192 + threadIdx.x] = 100 * steps + lanes;
+    int passed = 0;
+    if (waits) {
+        for (int step = 0; step < 3; ++step) {  // (one phase: once completed, every step sees it)
+            if (!mbar_wait(&lbar, 0u, status, limit)) {
+                leave_warp_loop(3 - step);
+                break;
+            }
+            ++passed;
+            __syncwarp();
+        }
+        out[192 + threadIdx.x] = 1000 * passed + 100 * steps + lanes;
+    } else {
+        complete(&lbar);
+    }
+    __syncthreads();
     int normal = 0, odds = 0;
     bool ok = true;
     for (int tile = 0; tile < 3; ++tile) {

@@ -28,7 +28,7 @@ def run(env, late, arrive, odd):
     torch.cuda.synchronize()
     # every lane took part in all its warp's sums; a lane whose wait gave up did nothing else
     seen = [3 if arrive == 1 or (arrive == 2 and t >= late) else 0 for t in range(96)]
-    assert out[192:].tolist() == [100 * s + 96 for s in seen]
+    assert out[192:].tolist() == [1100 * s + 96 for s in seen]
     return out[:192], geom.device_status(clear=True)
 
 
