@@ -21,10 +21,13 @@
 // in-plane coordinate q_b on every plane, and their q_z lie within 3 t drz voxels (0.8 at
 // the clinical isocentre), so they fall into two z-cells (a third or more where the rows are
 // coarser, decided per chunk): the thread interpolates the levels L_j they share once along b,
-// and a row at x cells above the lowest one is L_0 + sum_j sat(x - j) (L_{j+1} - L_j) — six
+// and a row at x cells above the lowest one is L_1 + sat(1 - x) (L_0 - L_1) + sat(x - 1) (L_2 - L_1) — six
 // shared loads and about 40 instructions for four samples, against sixteen loads and 90 for
-// four separate bilinear samples. The planes of a chunk are unrolled for two, for three and for
-// any number of cells: a test and a loop in every plane cost 8 % (clinical 7.87 -> 7.23 ms). L_0 is summed once for the four rows. Where a result is not
+// four separate bilinear samples. Both cells end at L_1, so that a level outside a row's own cell enters it
+// with an exact zero and leaves no rounding there, however large it is (started from L_0, a row two levels
+// away was off by 1e-7 of L_0: 4e-4 of its own value where L_0 is 10^4 times larger). With three cells and
+// more no level belongs to all of them, and each level gets its weight. The planes of a chunk are unrolled for two, for three and for
+// any number of cells: a test and a loop in every plane cost 8 % (clinical 7.87 -> 7.23 ms). L_1 is summed once for the four rows. Where a result is not
 // finite (a NaN or infinite voxel in a level that only some of the rows use) every ray is
 // summed again from its own samples. Sums run per chunk and then over chunks, which keeps the
 // rounding of a ray well below one long sum's: error against 64 bits 1.5e-7 at the clinical size
@@ -316,7 +319,7 @@ __global__ void __launch_bounds__(kThreads, forward_ctas(BW, ZH, kP))
                     const float *st = stages + s * SE;
                     const int base = -(ci.z0 * BW + ci.b0), cells = ci.cells;
                     const unsigned top = (unsigned)((ZH - cells) * BW - 2);
-                    // sums over the chunk of the lowest level, and of what each row adds to it
+                    // sums over the chunk of the level that all rows use, and of what each row adds to it
                     // (short partial sums: less rounding than one run over all planes)
                     float low = 0.f;
                     float2 part[2];
@@ -334,27 +337,45 @@ __global__ void __launch_bounds__(kThreads, forward_ctas(BW, ZH, kP))
                         const float2 va = make_float2(r[0], r[BW]), vb = make_float2(r[1], r[BW + 1]);
                         const float2 l01 = __ffma2_rn(make_float2(fb, fb), __ffma2_rn(va, make_float2(-1.f, -1.f), vb), va);
                         const float l2 = fmaf(fb, r[2 * BW + 1] - r[2 * BW], r[2 * BW]);
-                        const float j1 = jz + 1.f, e1 = l01.y - l01.x, e2 = l2 - l01.y;
-                        const float2 e11 = make_float2(e1, e1), e22 = make_float2(e2, e2);
-                        low += l01.x;
-                        part[0] = __ffma2_rn(make_float2(__saturatef(q0.x - jz), __saturatef(q0.y - jz)), e11, part[0]);
-                        part[1] = __ffma2_rn(make_float2(__saturatef(q1.x - jz), __saturatef(q1.y - jz)), e11, part[1]);
-                        part[0].y = fmaf(__saturatef(q0.y - j1), e2, part[0].y);
-                        part[1] = __ffma2_rn(make_float2(__saturatef(q1.x - j1), __saturatef(q1.y - j1)), e22, part[1]);
-                        float l = l2;
-                        auto more = [&](int m) {
-                            const float *rm = r + (m + 1) * BW;
-                            const float ln = fmaf(fb, rm[1] - rm[0], rm[0]), e = ln - l, jm = jz + (float)m;
-                            part[0].y = fmaf(__saturatef(q0.y - jm), e, part[0].y);
-                            const float2 e2m = make_float2(e, e);
-                            part[1] = __ffma2_rn(make_float2(__saturatef(q1.x - jm), __saturatef(q1.y - jm)), e2m, part[1]);
-                            l = ln;
-                        };
-                        if constexpr (known.value == 3) {
-                            more(2);
-                        } else if constexpr (known.value == 0) {
+                        const float j1 = jz + 1.f;
+                        if constexpr (known.value == 2) {
+                            // every row lies in a cell that has L_1 as one end
+                            const float e0 = l01.x - l01.y, e2 = l2 - l01.y;
+                            const float2 e00 = make_float2(e0, e0), e22 = make_float2(e2, e2);
+                            low += l01.y;
+                            part[0] = __ffma2_rn(make_float2(__saturatef(j1 - q0.x), __saturatef(j1 - q0.y)), e00, part[0]);
+                            part[1] = __ffma2_rn(make_float2(__saturatef(j1 - q1.x), __saturatef(j1 - q1.y)), e00, part[1]);
+                            part[0].y = fmaf(__saturatef(q0.y - j1), e2, part[0].y);
+                            part[1] = __ffma2_rn(make_float2(__saturatef(q1.x - j1), __saturatef(q1.y - j1)), e22, part[1]);
+                        } else {
+                            // level j weighs sat(x - j + 1) - sat(x - j): zero outside the row's own cell
+                            const float2 one = make_float2(1.f, 1.f), neg = make_float2(-1.f, -1.f);
+                            float2 s0 = make_float2(__saturatef(q0.x - jz), __saturatef(q0.y - jz));
+                            float2 s1 = make_float2(__saturatef(q1.x - jz), __saturatef(q1.y - jz));
+                            part[0] = __ffma2_rn(__ffma2_rn(s0, neg, one), make_float2(l01.x, l01.x), part[0]);
+                            part[1] = __ffma2_rn(__ffma2_rn(s1, neg, one), make_float2(l01.x, l01.x), part[1]);
+                            auto level = [&](float l, float j) {  // (the lowest row lies in the lowest cell)
+                                const float2 t0 = make_float2(0.f, __saturatef(q0.y - j));
+                                const float2 t1 = make_float2(__saturatef(q1.x - j), __saturatef(q1.y - j));
+                                part[0] = __ffma2_rn(__ffma2_rn(t0, neg, s0), make_float2(l, l), part[0]);
+                                part[1] = __ffma2_rn(__ffma2_rn(t1, neg, s1), make_float2(l, l), part[1]);
+                                s0 = t0;
+                                s1 = t1;
+                            };
+                            auto load = [&](int m) {
+                                const float *rm = r + m * BW;
+                                return fmaf(fb, rm[1] - rm[0], rm[0]);
+                            };
+                            level(l01.y, j1);
+                            level(l2, jz + 2.f);
+                            int m = 3;
+                            if constexpr (known.value == 0) {
 #pragma unroll 1
-                            for (int m = 2; m < cells; ++m) more(m);
+                                for (; m < cells; ++m) level(load(m), jz + (float)m);
+                            }
+                            const float l = load(m);
+                            part[0].y = fmaf(s0.y, l, part[0].y);
+                            part[1] = __ffma2_rn(s1, make_float2(l, l), part[1]);
                         }
                     };
                     // (planes past the volume are zero in the box)

@@ -86,3 +86,23 @@ def test_non_finite_voxels_reach_only_their_rays(name, value):
     far = w == 0
     assert bool(torch.isfinite(got[far]).all())
     assert float((got[far] - clean[far]).abs().max()) <= TOL * float(clean.abs().max())
+
+
+@pytest.mark.parametrize("name", ["box0", "box1_ragged", "box2", "box3", "box5_four_cells", "box6_five_cells"])
+@pytest.mark.parametrize("value", [1e2, 1e4, 1e6, 1e9])
+def test_large_voxels_leave_other_rays_alone(name, value):
+    """Large finite voxels (alternate z-slices of a block, so that rows which share levels lie on both
+    sides of them): a ray that gives them no weight keeps its value to a rounding of its own sum,
+    whatever they hold."""
+    geom = P.Geometry(CASES[name][0])
+    x = torch.as_tensor(I.random_volume((1,) + geom.vol_shape, 8), device="cuda").abs() + 0.1
+    clean = P.forward_project(geom, x)
+    nz, ny, nx = geom.vol_shape
+    hot = torch.zeros_like(x)
+    hot[0, nz // 4:3 * nz // 4:5, ny // 3:ny // 3 + 3, nx // 2:nx // 2 + 5] = 1.0
+    w = P.forward_project(geom, hot)      # the same sample positions
+    got = P.forward_project(geom, torch.where(hot > 0, torch.full_like(x, value), x))
+    far, near = w == 0, w > 0
+    assert int(near.sum()) > 100 and int(far.sum()) > 1000
+    # about a hundred positive samples, each rounded to 2^-24 of its value: the two sums may be grouped alike
+    assert float(((got[far] - clean[far]).abs() - 1e-6 * clean[far]).max()) <= 0.0
