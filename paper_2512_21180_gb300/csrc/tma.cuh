@@ -97,8 +97,8 @@ __device__ __forceinline__ void leave_warp_loop(int iterations) {
     for (; iterations > 0; --iterations) __syncwarp();
 }
 
-// What a CTA's threads found: whether one gave up a wait, and whether one saw something odd in
-// its data. Every thread gets the same answer. (A barrier's OR is a vote, not the OR of bits: two
+// What a CTA's threads found: whether one gave up a wait and, if none did, whether one saw something
+// odd in its data. Every thread gets the same answer. (A barrier's OR is a vote, not the OR of bits: two
 // questions take two votes, the second only where the first found anything.)
 struct CtaVote {
     bool gave_up, odd;
@@ -106,7 +106,7 @@ struct CtaVote {
 __device__ __forceinline__ CtaVote cta_vote(bool gave_up, bool odd) {
     if (!__syncthreads_or(gave_up || odd)) return CtaVote{false, false};
     const bool g = __syncthreads_or(gave_up) != 0;
-    return CtaVote{g, __syncthreads_or(odd) != 0};
+    return CtaVote{g, !g};
 }
 
 // 3D tiled TMA load of a box into shared memory, completion counted on `bar`.

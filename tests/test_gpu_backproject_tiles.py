@@ -81,3 +81,25 @@ def test_empty_projection_gives_exact_zeros():
     y[0, 3, 20, 50] = 1e6
     got, ref = P.back_project(geom, y), P.back_project(geom, y.double())
     assert bool((got[ref == 0] == 0).all())
+
+
+@pytest.mark.parametrize("name", ["fine_panel", "eight_per_part", "nu_113", "coarse_panel", "near_source"])
+@pytest.mark.parametrize("value", [1e2, 1e3, 1e4, 1e6, 1e9])
+def test_large_pixels_leave_other_voxels_alone(name, value):
+    """Large finite pixels on a positive background: a voxel that their rays give no weight keeps
+    its value. Columns that span more than a factor of 1024 (windows of up to four rows) are summed row by
+    row: 1e-5, the projector pair's bar, for 1e4 and more; so is 1e2 by its size. Just below the factor, a
+    prefix sum of 1024 windows rounds to 2^-24 of itself, 6e-5 of the smallest window, with a lever arm of up
+    to 26 rows in the interval's first moment: 1e-4 once the columns and angles of a voxel average it."""
+    geom = P.Geometry(CASES[name])
+    na, nv, nu = geom.proj_shape
+    y = torch.as_tensor(I.random_volume((1,) + geom.proj_shape, 9), device="cuda").abs() + 0.1
+    clean = P.back_project(geom, y)
+    hot = torch.zeros_like(y)
+    hot[0, :, nv // 4::max(1, nv // 3), nu // 5::max(1, nu // 4)] = 1.0
+    w = P.back_project(geom, hot)
+    got = P.back_project(geom, torch.where(hot > 0, torch.full_like(y, value), y))
+    far = (w == 0) & (P.back_project(geom, hot.double()) == 0) & (clean > 0.05 * clean.max())
+    assert int(far.sum()) > 300 and int((w > 0).sum()) > 50
+    tol = 1e-4 if value == 1e3 else 1e-5
+    assert float(((got[far] - clean[far]).abs() / clean[far]).max()) <= tol
