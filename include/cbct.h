@@ -282,6 +282,8 @@ int cbct_fdk_pad(const cbct_geom *g);
  * tau = du sid / sdd (tau h(0) = 1/(4 tau), tau h(odd j) = -1/(pi^2 j^2 tau)), then
  * vol(P) (+)= (2 pi / n_angles) sum_k (sid / U_k)^2 q_k(u_k(P), v_k(P)) with bilinear
  * sampling (zero off the extended panel), U_k the depth of P along the central ray.
+ * A filtered row's rounding is relative to that row's own largest value (about 1e-7 of it), and an
+ * empty row stays exactly zero.
  * Scratch: about batch n_angles nv (nu + pad) floats, twice
  * that when the rows are filtered directly (nu + pad <= 256 or > 2048, or fewer than 1024
  * rows), and up to 16 partial volumes for small volumes. */

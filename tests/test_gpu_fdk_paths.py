@@ -96,3 +96,46 @@ def test_a_bad_row_leaves_its_partner_alone(O, rows, value):
         for iv in rows:
             near |= (fv - iv).abs() < 0.9
         assert int((~torch.isfinite(got[near])).sum()) > 50
+
+
+def detector_rows(geom, g, k):
+    """Detector row coordinate of every voxel at angle k."""
+    z, yy, x = (torch.arange(n, device="cuda", dtype=torch.float64) - 0.5 * (n - 1) for n in geom.vol_shape)
+    th = 2 * np.pi * k / g["n_angles"]
+    U = 1000.0 - 4.0 * (x[None, :] * np.cos(th) + yy[:, None] * np.sin(th))
+    fv = (1536.0 / U)[None] * (4.0 * z)[:, None, None] - g["v_offset"]
+    return (fv / g["dv"] + 0.5 * (g["nv"] - 1))[None]
+
+
+@pytest.mark.parametrize("name", ["fft1024", "fft2048_offset", "fft4096"])
+@pytest.mark.parametrize("large", [12, 13])
+@pytest.mark.parametrize("factor", [1e3, 1e6, 1e9, 1e30])
+def test_rows_round_to_their_own_size(name, large, factor):
+    """Rows 12 and 13 share a transform; one of them is larger by a factor. The voxels on the other
+    row's side do not see it and keep what they get beside an empty row, to the transform's rounding of
+    their own row (about 11 passes of 2^-24 on values three times the largest output: 2e-6)."""
+    g, k = CASES[name], 5
+    geom = P.Geometry(g)
+    y = torch.zeros((1,) + geom.proj_shape, device="cuda")
+    y[0, k] = to_gpu(I.random_volume(geom.proj_shape[1:], 6)).abs() + 0.1
+    alone, beside = y.clone(), y.clone()
+    alone[0, k, large] = 0.0
+    beside[0, k, large] *= factor
+    want, got = ops.fdk(geom, alone), ops.fdk(geom, beside)
+    fv = detector_rows(geom, g, k)
+    far = (fv < large - 1.01) | (fv > large + 1.01)
+    other = far & ((fv - (25 - large)).abs() < 0.9)   # voxels that see the partner
+    assert int(far.sum()) > 1000 and int(other.sum()) > 50
+    assert float((got[far] - want[far]).abs().max()) <= 2e-6 * float(want.abs().max())
+
+
+@pytest.mark.parametrize("name", ["fft1024", "fft4096"])
+def test_an_empty_row_stays_empty_beside_its_partner(name):
+    g, k = CASES[name], 5
+    geom = P.Geometry(g)
+    y = torch.zeros((1,) + geom.proj_shape, device="cuda")
+    y[0, k, 12] = to_gpu(I.random_volume((geom.proj_shape[2],), 6)).abs() + 0.1
+    got, fv = ops.fdk(geom, y), detector_rows(geom, g, k)
+    partner = (fv > 13.01) & (fv < 13.9)
+    assert int(partner.sum()) > 100 and int((got != 0).sum()) > 100
+    assert bool((got[partner] == 0).all())
