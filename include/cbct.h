@@ -117,11 +117,14 @@ int cbct_forward_config(const cbct_geom *g, int *cfg, double *need_b, double *ne
  * accumulate = 0 overwrites proj, 1 adds to it. FP32 in, FP32 accumulation.
  * batch >= 1; batch * n_angles <= 65535. Scratch: a plane-major copy of the
  * volumes (batch * nx * ny * nz floats, rows padded to 4; a second one when nx is not a
- * multiple of 4 or vol not on 16 bytes), from the stream-ordered pool; none for calls of
- * at most 2^20 rays times planes. Errors: CBCT_EINVAL (before any launch) for a NULL pointer,
- * batch < 1, accumulate not 0 or 1, batch * n_angles > 65535 or a current device
- * other than the geometry's; CBCT_ENOMEM when the scratch cannot be allocated;
- * CBCT_ECUDA for a failed launch. */
+ * multiple of 4 or vol not on 16 bytes), from the stream-ordered pool. A kernel without
+ * scratch serves calls of at most 2^20 rays times planes (batch included), panels too coarse
+ * for a shared-memory box, and calls whose scratch cannot be allocated; it adds a ray's samples in
+ * another order, so a volume's result in a batch can differ from its single-volume result by FP32
+ * summation order (the same call always gives the same bits while its scratch is to be had). A voxel that
+ * a ray gives no weight leaves no rounding in it, however large it is. Errors: CBCT_EINVAL (before any
+ * launch) for a NULL pointer, batch < 1, accumulate not 0 or 1, batch * n_angles > 65535 or a
+ * current device other than the geometry's; CBCT_ECUDA for a failed launch. */
 int forward_project(const cbct_geom *g, const float *vol, float *proj, int batch, int accumulate,
                     void *stream);
 

@@ -110,28 +110,37 @@ __device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *map, i
 
 // ---- plane-major copies ----------------------------------------------------------------
 
+// (both: slices z of all items go round the grid, whose z and y extents end at 65535)
 // T_y[b][y][z][x] = V[b][z][y][x]   (row pitch py >= nx)
-__global__ void k_planes_y(const float *__restrict__ V, float *__restrict__ T, int nx, int ny, int nz, int py) {
-    const int y = blockIdx.x, z = blockIdx.y, b = blockIdx.z;
-    const float *src = V + (((long long)b * nz + z) * ny + y) * nx;
-    float *dst = T + (((long long)b * ny + y) * nz + z) * py;
-    for (int x = threadIdx.x; x < nx; x += blockDim.x) dst[x] = src[x];
+__global__ void k_planes_y(const float *__restrict__ V, float *__restrict__ T, int nx, int ny, int nz, long long slices,
+                           int py) {
+    const int y = blockIdx.x;
+    for (long long s = blockIdx.y; s < slices; s += gridDim.y) {
+        const long long b = s / nz, z = s - b * nz;
+        const float *src = V + (s * ny + y) * nx;
+        float *dst = T + ((b * ny + y) * nz + z) * py;
+        for (int x = threadIdx.x; x < nx; x += blockDim.x) dst[x] = src[x];
+    }
 }
 
 // T_x[b][x][z][y] = V[b][z][y][x]   (row pitch px >= ny), 32x32 tiles through smem
-__global__ void k_planes_x(const float *__restrict__ V, float *__restrict__ T, int nx, int ny, int nz, int px) {
+__global__ void k_planes_x(const float *__restrict__ V, float *__restrict__ T, int nx, int ny, int nz, long long slices,
+                           int px) {
     __shared__ float tile[32][33];
     const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 32;
-    const int z = blockIdx.z % nz, b = blockIdx.z / nz;
-    const float *src = V + ((long long)b * nz + z) * ny * (long long)nx;
-    for (int j = threadIdx.y; j < 32; j += blockDim.y) {
-        const int y = y0 + j, x = x0 + threadIdx.x;
-        tile[j][threadIdx.x] = (y < ny && x < nx) ? src[(long long)y * nx + x] : 0.0f;
-    }
-    __syncthreads();
-    for (int j = threadIdx.y; j < 32; j += blockDim.y) {
-        const int x = x0 + j, y = y0 + threadIdx.x;
-        if (x < nx && y < ny) T[(((long long)b * nx + x) * nz + z) * px + y] = tile[threadIdx.x][j];
+    for (long long s = blockIdx.z; s < slices; s += gridDim.z) {
+        const long long b = s / nz, z = s - b * nz;
+        const float *src = V + s * ny * (long long)nx;
+        for (int j = threadIdx.y; j < 32; j += blockDim.y) {
+            const int y = y0 + j, x = x0 + threadIdx.x;
+            tile[j][threadIdx.x] = (y < ny && x < nx) ? src[(long long)y * nx + x] : 0.0f;
+        }
+        __syncthreads();
+        for (int j = threadIdx.y; j < 32; j += blockDim.y) {
+            const int x = x0 + j, y = y0 + threadIdx.x;
+            if (x < nx && y < ny) T[((b * nx + x) * nz + z) * px + y] = tile[threadIdx.x][j];
+        }
+        __syncthreads();
     }
 }
 
@@ -454,15 +463,20 @@ struct FwdCfg {
 };
 static const FwdCfg kCfgs[] = {{28, 14, 8}, {32, 16, 8}, {36, 18, 8}, {40, 24, 4}, {48, 28, 4}, {64, 36, 4}, {96, 48, 2}};
 
+// Shared memory of the staged kernel: two boxes, their barriers, the chunk list, the abort flag.
+static size_t staged_smem(const GeomDev &d, const FwdCfg &c) {
+    const size_t chunks = (std::max(d.n[0], d.n[1]) + c.np - 1) / c.np;
+    return 128 + (size_t)kStages * c.np * c.zh * c.bw * 4 + 2 * kStages * 8 + chunks * sizeof(ChunkInfo) + sizeof(int);
+}
+constexpr size_t kStagedSmemMax = 227 * 1024;
+
 template <int BW, int ZH, int NP>
 static int launch_cfg(const cbct_geom *g, const CUtensorMap &mx, const CUtensorMap &my, const PlaneView &vx,
                       const PlaneView &vy, float *proj, int batch, int accumulate, cudaStream_t st) {
     static_assert(BW % 4 == 0 && BW <= 256 && ZH <= 256, "TMA box");
     const GeomDev &d = g->dev;
-    const int maxch = (std::max(d.n[0], d.n[1]) + NP - 1) / NP;
-    const size_t smem =
-        128 + (size_t)kStages * NP * ZH * BW * 4 + 2 * kStages * 8 + (size_t)maxch * sizeof(ChunkInfo) + sizeof(int);
     auto kern = k_forward_tma<BW, ZH, NP>;
+    const size_t smem = staged_smem(d, FwdCfg{BW, ZH, NP});
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail(e, "forward_project: smem attribute");
     dim3 grd((d.nu + kTU - 1) / kTU, (d.nv + kTV - 1) / kTV, d.na * batch);
@@ -476,32 +490,40 @@ static int launch_cfg(const cbct_geom *g, const CUtensorMap &mx, const CUtensorM
 // (2^24.6) 88 against 38.
 constexpr long long kDirectSamples = 1 << 20;
 
-// Returns 1 if the staged kernel handled the call, 0 if the caller should use the
-// direct kernel, negative on error.
+// Returns 1 if the staged kernel handled the call, 0 if the caller should use the direct kernel
+// (small calls, boxes or chunk lists that do not fit, no memory for the plane copies: the direct kernel
+// needs none), negative on error.
 int forward_staged(const cbct_geom *g, const float *vol, float *proj, int batch, int accumulate, cudaStream_t st) {
     const GeomDev &d = g->dev;
     const int nx = d.n[0], ny = d.n[1], nz = d.n[2];
     if (g->fwd_cfg < 0 || (long long)batch * d.na * d.nv * d.nu * std::max(nx, ny) <= kDirectSamples) return 0;
-    const long long nvox = (long long)nx * ny * nz;
+    const FwdCfg cf = kCfgs[g->fwd_cfg];
+    if (staged_smem(d, cf) > kStagedSmemMax) return 0;
+    const long long nvox = (long long)nx * ny * nz, slices = (long long)nz * batch;
     // y planes are read from the volume itself when its rows start on 16 bytes (a TMA stride)
     const bool copy_y = (nx & 3) != 0 || (reinterpret_cast<uintptr_t>(vol) & 15) != 0;
     const int px = (ny + 3) & ~3, py = (nx + 3) & ~3;
     const long long ex = (long long)batch * nx * nz * px, ey = copy_y ? (long long)batch * ny * nz * py : 0;
     float *buf = nullptr;
-    CBCT_CUDA_TRY(scratch_alloc((void **)&buf, sizeof(float) * (ex + ey), st));
+    const cudaError_t ea = scratch_alloc((void **)&buf, sizeof(float) * (ex + ey), st);
+    if (ea == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        return 0;
+    }
+    CBCT_CUDA_TRY(ea);
     float *tx = buf, *ty = buf + ex;
     const PlaneView vx{tx, (long long)nx * nz * px, (long long)nz * px, px};
     const PlaneView vy = copy_y ? PlaneView{ty, (long long)ny * nz * py, (long long)nz * py, py}
                                 : PlaneView{vol, nvox, nx, (long long)nx * ny};
     int rc = 0;
     {
-        dim3 gx((nx + 31) / 32, (ny + 31) / 32, nz * batch);
-        k_planes_x<<<gx, dim3(32, 8), 0, st>>>(vol, tx, nx, ny, nz, px);
-        if (copy_y) k_planes_y<<<dim3(ny, nz, batch), 128, 0, st>>>(vol, ty, nx, ny, nz, py);
+        const unsigned gz = (unsigned)std::min<long long>(slices, 65535);
+        dim3 gx((nx + 31) / 32, (ny + 31) / 32, gz);
+        k_planes_x<<<gx, dim3(32, 8), 0, st>>>(vol, tx, nx, ny, nz, slices, px);
+        if (copy_y) k_planes_y<<<dim3(ny, gz), 128, 0, st>>>(vol, ty, nx, ny, nz, slices, py);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) rc = cuda_fail(e, "forward_project: plane copies");
     }
-    const FwdCfg cf = kCfgs[g->fwd_cfg];
     CUtensorMap mx, my;
     if (rc == 0) {
         auto encode = [&](CUtensorMap *m, const PlaneView &v, int nb, int np) {

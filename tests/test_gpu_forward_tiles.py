@@ -57,6 +57,21 @@ def test_boxes_match_fp64(name, batch):
     assert geom.device_status() == 0
 
 
+@pytest.mark.parametrize("nx", [16, 17])
+@pytest.mark.parametrize("du,cfg", [(3.2, None), (4.5, 4)])
+def test_more_slices_than_a_grid_holds(du, cfg, nx):
+    """257 volumes of 256 slices (65,792): more than a grid's z extent, on a fine panel and on one
+    whose box is among the coarse ones; items against the FP64 instantiation."""
+    geom = P.Geometry(I.scaled(T, n=(nx, 16, 256), vox=(4.0, 4.0, 4.0), nu=31, nv=33, du=du, dv=1.1 * du, n_angles=5))
+    c = ctypes.c_int()
+    _lib.check(_lib.load().cbct_forward_config(geom.handle, ctypes.byref(c), None, None))
+    assert c.value >= 0 and (cfg is None or c.value == cfg)
+    x = torch.as_tensor(I.random_volume((257,) + geom.vol_shape, 23), device="cuda")
+    got = P.forward_project(geom, x)
+    for b in (0, 128, 255, 256):
+        check(got[b:b + 1], P.forward_project(geom, x[b:b + 1].double()))
+
+
 def test_volume_rows_off_16_bytes():
     """A contiguous volume at an odd element offset of a larger buffer (x rows of 64 voxels)."""
     geom = P.Geometry(CASES["box0"][0])
