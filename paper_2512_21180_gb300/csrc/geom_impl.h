@@ -68,6 +68,7 @@ int conv_pack_jobs(const ConvPackJob *jobs, int njobs, long long max_nelem, cons
 // back_project_noalloc's fixed scratch array, so that the module holding the array is
 // loaded, and the array placed, when the geometry is made.
 int projector_prime(int dev);
+int forward_prime();  // (its part for the staged forward kernels)
 // Ray tile of the staged forward (columns x rows).
 constexpr int kForwardTileCols = 32, kForwardTileRows = 16;
 // Staged (TMA) forward: returns 1 if it ran, 0 if the direct kernel must be used.

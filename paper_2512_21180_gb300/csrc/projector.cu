@@ -982,7 +982,8 @@ int projector_prime(int dev) {
     float *p = nullptr;
     for (auto kern : {k_backproject_seg<1>, k_backproject_seg<4>})
         CBCT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem3));
-    return noalloc_scratch(dev, &p);
+    const int rc = forward_prime();
+    return rc ? rc : noalloc_scratch(dev, &p);
 }
 
 }  // namespace cbct

@@ -477,8 +477,6 @@ static int launch_cfg(const cbct_geom *g, const CUtensorMap &mx, const CUtensorM
     const GeomDev &d = g->dev;
     auto kern = k_forward_tma<BW, ZH, NP>;
     const size_t smem = staged_smem(d, FwdCfg{BW, ZH, NP});
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_fail(e, "forward_project: smem attribute");
     dim3 grd((d.nu + kTU - 1) / kTU, (d.nv + kTV - 1) / kTV, d.na * batch);
     kern<<<grd, kThreads, smem, st>>>(mx, my, d, vx, vy, proj, accumulate, g->status);
     CBCT_LAUNCH_CHECK("forward_project (staged) launch");
@@ -548,6 +546,15 @@ int forward_staged(const cbct_geom *g, const float *vol, float *proj, int batch,
     }
     cudaFreeAsync(buf, st);
     return rc == 0 ? 1 : rc;
+}
+
+// Shared-memory limits of the staged kernels on the current device (once per geometry: a limit set by
+// each call for its own volume could be lowered by another thread's call before the launch).
+int forward_prime() {
+    for (auto kern : {k_forward_tma<28, 14, 8>, k_forward_tma<32, 16, 8>, k_forward_tma<36, 18, 8>, k_forward_tma<40, 24, 4>,
+                      k_forward_tma<48, 28, 4>, k_forward_tma<64, 36, 4>, k_forward_tma<96, 48, 2>})
+        CBCT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStagedSmemMax));
+    return 0;
 }
 
 // Pick the smallest box that holds a tile's footprint over one chunk of np planes (need + (np -

@@ -72,6 +72,31 @@ def test_more_slices_than_a_grid_holds(du, cfg, nx):
         check(got[b:b + 1], P.forward_project(geom, x[b:b + 1].double()))
 
 
+def test_threads_with_geometries_of_one_box():
+    """Two volumes of different length share a kernel whose shared memory follows the length."""
+    import threading
+    geoms = [P.Geometry(scan((n, 60, 40), 4.0, 130, 70, 1.2, 1.2)) for n in (64, 66)]
+    xs = [torch.as_tensor(I.random_volume((1,) + g.vol_shape, 3), device="cuda") for g in geoms]
+    want = [P.forward_project(g, x) for g, x in zip(geoms, xs)]
+    torch.cuda.synchronize()
+    bad = []
+
+    def work(i):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                outs = [P.forward_project(geoms[i], xs[i]) for _ in range(100)]
+                torch.cuda.current_stream().synchronize()
+                if not all(torch.equal(o, want[i]) for o in outs):
+                    bad.append(i)
+        except Exception as e:  # (a refused launch)
+            bad.append(e)
+
+    ts = [threading.Thread(target=work, args=(i % 2,)) for i in range(4)]
+    [t.start() for t in ts]
+    [t.join() for t in ts]
+    assert not bad
+
+
 def test_volume_rows_off_16_bytes():
     """A contiguous volume at an odd element offset of a larger buffer (x rows of 64 voxels)."""
     geom = P.Geometry(CASES["box0"][0])
