@@ -610,12 +610,19 @@ extern "C" int cbct_fdk(const cbct_geom *g, const float *proj, float *vol, int b
     const long long ctas = (long long)((d.nx + 31) / 32) * ((d.ny + 7) / 8) * nzr * batch;
     int nparts = (int)std::max<long long>(1, std::min<long long>({16, d.n_angles / 8, 8LL * sm_count() / ctas}));
     while (nparts > 1 && (long long)nzr * batch * nparts > 65535) --nparts;
-    const long long nvol = (long long)batch * d.nx * d.ny * d.nz, npart = nparts > 1 ? nparts * nvol : 0;
+    const long long nvol = (long long)batch * d.nx * d.ny * d.nz;
     // q: filtered rows, zero-bordered [batch na][nv + 2][nue + 2]; q0: weighted extended rows [rows][nue] for
     // the direct filter
     const long long nq0 = nfft ? 0 : padded(rows * nue), nq = padded((long long)batch * d.n_angles * (d.nv + 2) * (nue + 2));
     float *q0 = nullptr, *q = nullptr, *w = nullptr;
-    CBCT_CUDA_TRY(scratch_alloc((void **)&q0, sizeof(float) * (nq0 + nq + padded(d.nu) + nfft + npart), st));
+    const long long fixed = nq0 + nq + padded(d.nu) + nfft;
+    cudaError_t ea = scratch_alloc((void **)&q0, sizeof(float) * (fixed + (nparts > 1 ? nparts * nvol : 0)), st);
+    if (ea == cudaErrorMemoryAllocation && nparts > 1) {  // without the parts' volumes
+        cudaGetLastError();
+        nparts = 1;
+        ea = scratch_alloc((void **)&q0, sizeof(float) * fixed, st);
+    }
+    CBCT_CUDA_TRY(ea);
     q = q0 + nq0;
     w = q + nq;
     float *H = w + padded(d.nu), *partial = H + nfft;
