@@ -76,3 +76,44 @@ def test_calls_in_a_graph():
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(f, want[0]) and torch.equal(b, want[1])
+
+
+LAST_ONE = """
+import torch
+from paper_2512_21180_gb300 import inputs as I
+from paper_2512_21180_gb300 import projector as P
+a, b = P.Geometry(I.geometry("clinical")), P.Geometry(I.geometry("tiny16"))
+y = torch.rand((2,) + a.proj_shape, device="cuda")      # 0.63 GB of weighted projections
+out = torch.empty((2,) + a.vol_shape, device="cuda")
+P.back_project(b, torch.zeros((1,) + b.proj_shape, device="cuda"))   # loads the kernels
+torch.cuda.synchronize()
+start = torch.cuda.mem_get_info()[0]
+def held():
+    torch.cuda.synchronize()
+    return (start - torch.cuda.mem_get_info()[0]) >> 20
+P.back_project(a, y, out=out)
+print(held())
+a.close()
+print(held())
+b.close()
+print(held())
+c = P.Geometry(I.geometry("clinical"))
+P.back_project(c, y, out=out)
+print(held())
+c.close()
+print(held())
+"""
+
+
+def test_the_last_geometry_gives_the_memory_back():
+    """In a process of its own (no other geometries): MiB held after a call, after closing one of two
+    geometries, after closing the last, and the same again with a new one."""
+    import subprocess
+    import sys
+    r = subprocess.run([sys.executable, "-c", LAST_ONE], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+    call, one_left, none_left, call2, none_left2 = (int(v) for v in r.stdout.split())
+    assert 512 <= call <= 1024 + 64
+    assert 512 <= one_left <= 1024 + 64
+    assert none_left <= 64 and none_left2 <= 64
+    assert 512 <= call2 <= 1024 + 64
