@@ -377,3 +377,40 @@ def test_conv_weight_gradient_wide(L, taps3d, dims, cin, cout, cpin, cpout):
     ref_dw = wr.grad.reshape(cout, cin, -1).permute(0, 2, 1) + 0.5
     assert rel_l2_t(dw.double().cpu(), ref_dw) <= 1e-5
     assert rel_l2_t(db.double().cpu(), br.grad + 0.5) <= 1e-5
+
+
+@pytest.mark.parametrize("taps3d,nimg,dims,cin,cout,cpin,cpout", [
+    # 5 to 6 tiles a CTA and depth tap, ragged in w and h: carries of the tile step, three segments
+    (1, 2, (9, 30, 130), 32, 32, 32, 32), (1, 2, (5, 41, 300), 6, 32, 8, 32), (1, 3, (7, 31, 129), 32, 5, 32, 8),
+    # 3 to 4 tiles a segment of two depth planes; as many tiles as CTAs and one more
+    (1, 1, (2, 303, 200), 20, 12, 32, 16), (1, 1, (1, 202, 128), 32, 32, 32, 32), (1, 1, (1, 204, 128), 32, 32, 32, 32),
+    # 2-D: two tiles and more a CTA
+    (0, 9, (77, 140), 32, 32, 32, 32), (0, 5, (63, 260), 7, 32, 8, 32),
+    # 13 tiles a segment of a 3-D layer
+    (1, 1, (64, 128, 128), 32, 32, 32, 32)])
+def test_conv_weight_gradient_many_tiles(L, taps3d, nimg, dims, cin, cout, cpin, cpout):
+    """Weight and bias gradients over several tiles a CTA, against 64 bits (on the GPU). Bound: one FP32
+    accumulation over 27 tiles measures 4.0e-6, over 81 tiles 9.3e-6; no segment here has more than 14."""
+    from oracle import lpd_ref as R
+    gen = torch.Generator().manual_seed(29)
+    x = R.bf16(torch.randn((nimg, cin) + dims, generator=gen, dtype=torch.float64))
+    dy = R.bf16(torch.randn((nimg, cout) + dims, generator=gen, dtype=torch.float64))
+    shape = (cout, cin) + (3,) * len(dims)
+    xg, dyg = x.cuda(), dy.cuda()
+    pad = torch.nn.functional.pad(xg, (1, 1) * len(dims))
+    ref = torch.empty(shape, dtype=torch.float64, device="cuda")
+    for tap in np.ndindex(*shape[2:]):   # dW[co, ci, tap] = sum over pixels of dY[co] X[ci, shifted by tap]
+        win = pad[(slice(None), slice(None)) + tuple(slice(t, t + n) for t, n in zip(tap, dims))]
+        ref[(slice(None), slice(None)) + tap] = torch.einsum("ncp,ndp->cd", dyg.flatten(2), win.flatten(2))
+    D, H, W = dims if taps3d else (1,) + dims
+    dw = torch.full((cout, 27 if taps3d else 9, cin), float("nan"), device="cuda")
+    db = torch.full((cout,), float("nan"), device="cuda")
+    x_cl, dy_cl = to_cl(x, cpin), to_cl(dy, cpout)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    L.check(L.load().cbct_conv_wgrad(x_cl.data_ptr(), cpin, cin, dy_cl.data_ptr(), cpout, cout, nimg, D, H, W,
+                                     taps3d, dw.data_ptr(), db.data_ptr(), 0, status.data_ptr(),
+                                     torch.cuda.current_stream().cuda_stream), "wgrad")
+    torch.cuda.synchronize()
+    assert status.item() == 0
+    assert rel_l2_t(dw.double(), ref.reshape(cout, cin, -1).permute(0, 2, 1)) <= 4e-6
+    assert rel_l2_t(db.double(), dyg.sum(dim=(0,) + tuple(range(2, dyg.dim())))) <= 4e-6
