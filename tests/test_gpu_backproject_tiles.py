@@ -103,3 +103,16 @@ def test_large_pixels_leave_other_voxels_alone(name, value):
     assert int(far.sum()) > 300 and int((w > 0).sum()) > 50
     tol = 1e-4 if value == 1e3 else 1e-5
     assert float(((got[far] - clean[far]).abs() / clean[far]).max()) <= tol
+
+
+@pytest.mark.parametrize("name", ["many_angles", "eight_per_part", "nu_113", "near_source"])
+def test_smooth_projections_to_a_few_roundings(name):
+    """On smooth projections a voxel is a sum of short FP32 sums: measured 1.6e-7 to 3.5e-7 of the norm on
+    scans; 1e-6 tells a longer sum or a lost bit."""
+    geom = P.Geometry(CASES[name])
+    na, nv, nu = geom.proj_shape
+    k, v, u = (torch.linspace(-1, 1, n, device="cuda", dtype=torch.float64) for n in (na, nv, nu))
+    p = 3.0 * torch.exp(-u[None, None] ** 2 - v[None, :, None] ** 2) * (1.0 + 0.2 * torch.cos(9.0 * k))[:, None, None]
+    p = p.float()[None].contiguous()
+    got, ref = P.back_project(geom, p), P.back_project(geom, p.double())
+    assert float((got.double() - ref).norm()) <= 1e-6 * float(ref.norm())
