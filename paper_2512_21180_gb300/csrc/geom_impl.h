@@ -33,6 +33,8 @@ int operator_norm(cbct_geom *g, int iters, double *out);
 // P^T (colw[u] * proj): adjoint of a column-weighted projection (colw: [nu] device).
 int back_project_colw(const cbct_geom *g, const float *proj, const float *colw, float *vol, int batch, int accumulate,
                       cudaStream_t st);
+// vol (+)= sum over parts of partial[part][n], in part order (the caller checks the launch).
+void sum_parts(const float *partial, int nparts, long long n, float *vol, int accumulate, cudaStream_t st);
 // cbct_conv with the residual epilogue reading its old state from state_in (which may
 // equal state) and writing state = state_in + conv (state = conv without reading
 // state_in when zero_state_in; state_in - conv with ssub). packed: the layer's B operand

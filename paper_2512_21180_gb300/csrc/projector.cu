@@ -694,6 +694,11 @@ __global__ void k_sum_parts(const float *__restrict__ partial, int nparts, long 
     }
 }
 
+void sum_parts(const float *partial, int nparts, long long n, float *vol, int accumulate, cudaStream_t st) {
+    const int gs = (int)std::min<long long>(8LL * sm_count(), (n + 255) / 256);
+    k_sum_parts<<<gs, 256, 0, st>>>(partial, nparts, n, vol, accumulate);
+}
+
 // ---- sample count -----------------------------------------------------------------
 
 __global__ void __launch_bounds__(256) k_count(GeomDev g, unsigned long long *total) {
@@ -820,8 +825,7 @@ static int backward_segments(const cbct_geom *g, const float *proj, float *vol, 
                                                                            g->status);
         e = cudaGetLastError();
         if (e == cudaSuccess && nparts > 1) {
-            const int gs = (int)std::min<long long>(8LL * sm_count(), (nvol + 255) / 256);
-            k_sum_parts<<<gs, 256, 0, st>>>(partial, nparts, nvol, vol, accumulate);
+            sum_parts(partial, nparts, nvol, vol, accumulate, st);
             e = cudaGetLastError();
         }
     }

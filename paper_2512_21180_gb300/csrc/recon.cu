@@ -462,16 +462,6 @@ __global__ void __launch_bounds__(256, 4) k_fdk_backproject(const float *__restr
     }
 }
 
-// vol (+)= sum of the parts' volumes, in part order
-__global__ void k_fdk_sum(const float *__restrict__ partial, int nparts, long long n, float *__restrict__ vol,
-                          int accumulate) {
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        float s = accumulate ? vol[e] : 0.f;
-        for (int p = 0; p < nparts; ++p) s += partial[(long long)p * n + e];
-        vol[e] = s;
-    }
-}
-
 // ---- PDHG-TV pieces -------------------------------------------------------------------
 
 // z1 <- (z1 + sigma (p - y)) / (1 + sigma)
@@ -652,7 +642,7 @@ extern "C" int cbct_fdk(const cbct_geom *g, const float *proj, float *vol, int b
             (float)d.vox[2], (float)d.center[0], (float)d.center[1], (float)d.center[2], (float)d.sid, (float)d.sdd,
             (float)(1.0 / d.du), (float)(1.0 / d.dv), (float)d.u_offset, (float)d.v_offset, nparts > 1 ? 0 : accumulate,
             nparts);
-        if (nparts > 1) k_fdk_sum<<<grid1(nvol), 256, 0, st>>>(partial, nparts, nvol, vol, accumulate);
+        if (nparts > 1) sum_parts(partial, nparts, nvol, vol, accumulate, st);
         e = cudaGetLastError();
     }
     cudaFreeAsync(q0, st);
