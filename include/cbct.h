@@ -132,10 +132,10 @@ int forward_project(const cbct_geom *g, const float *vol, float *proj, int batch
  * forward_project (same rays, planes and bilinear weights), computed as an
  * atomic-free voxel-driven gather. Scratch: batch * n_angles * nv * nu floats (nu
  * rounded up to 4; the ray-weighted projections, plus up to 16 partial volumes when
- * small volumes split the angles), from the stream-ordered pool. The rounding of a pixel stays
- * within its detector column, and there within the voxels its ray touches and those whose pixels are
- * not smaller than it by a factor of about 10^3: a voxel that a larger (or infinite, or NaN) pixel
- * does not touch keeps its value. A kernel that gives up
+ * small volumes split the angles), from the stream-ordered pool. A pixel leaves
+ * its rounding within its own detector column only, and there in no voxel that its ray does not touch
+ * and whose pixels are smaller by more than about 10^3 (it may be infinite or NaN; contrast is looked
+ * for from four rows to four rows of the panel). A kernel that gives up
  * waiting on its loads reports through cbct_device_status. The split follows the size of the
  * grid (volume and batch), so a volume's result in a batch can differ from its
  * single-volume result by FP32 summation order; a given geometry and batch size

@@ -275,24 +275,24 @@ __global__ void __launch_bounds__(256) k_backproject(GeomDev g, const T *__restr
 // sum (row - h) p) down each column, and every interval is the difference of two entries:
 // 10 instructions instead of a run of predicated row loads (3 to 5 rows per interval at
 // these magnifications); boundaries, shares and sums of two voxels go through packed FP32
-// instructions (12, one voxel at a time, with the same results: clinical 9.02 against 8.82 ms). The sums start at the tile's middle row h and run outwards, so
+// instructions (12, one voxel at a time, with the same results: clinical 9.02 against 8.82 ms). The
+// sums start at the tile's middle row h and run outwards, so
 // they span at most half a tile (26 rows) of one column: FP32 rounding stays that of a
 // short sum, and the measured error against 64 bits is the row-by-row kernel's (clinical
-// 3.3e-7 against 3.5e-7). Bounded by instruction issue (62 % of the issue slots; the rest
+// 3.3e-7 against 3.5e-7). Bounded by instruction issue (66 % of the issue slots; the rest
 // mostly the two barriers of a tile, 24 % of the stalls): about 3/4 of the instructions are the
-// intervals, 1/8 the prefix sums. Back projection by CUDA events, row by row -> now:
-// clinical 17.4 -> 8.82 ms, 2 x 128^3 / 200 angles 3.79 -> 1.58 ms, 181 x 167 x 93 / 150 angles
-// 4.12 -> 1.19 ms, 64^3 / 64 angles 126 -> 60 us.
+// intervals, 1/6 the prefix sums. Back projection by CUDA events, row by row -> now:
+// clinical 17.4 -> 9.73 ms, 2 x 128^3 / 200 angles 3.79 -> 1.70 ms, 64^3 / 64 angles 126 -> 54 us.
 //
 // A prefix sum keeps the rounding of every row on its way, so a column half that is not finite or
-// spans too wide a range (kWideRatio) is summed row by row instead, over the same intervals: a large,
+// spans too wide a range (kWideLog2) is summed row by row instead, over the same intervals: a large,
 // infinite or NaN pixel reaches the voxels its ray touches and no others. Below the factor the
 // differences round to little more than what the positions do (largest error of a voxel that pixels 10^3 times
 // their background do not touch, 100 angles: 8.6e-6 of its value against 3.7e-6 without them; with prefix
-// sums everywhere 8e-5 at 10^4 and 6e-3 at 10^6). Such columns lie at the edges of the body: 0.1 % of the column
-// halves of a phantom's projections, and with noise 0.05 beside sums of 10 they cost the clinical adjoint 4 %.
-// They are read from the landing box, so the next one is sent for after them. Watching the windows costs
-// every tile 1 %. A brick
+// sums everywhere 8e-5 at 10^4 and 6e-3 at 10^6). Such columns lie
+// at the edges of the body, where a tile's middle is inside it: 0.1 % of the column halves of a phantom's
+// projections, which cost the clinical adjoint 6 %.
+// They are read from the landing box, so the next one is sent for after them. A brick
 // whose footprint exceeds the tile takes several tiles per angle: the intervals are linear in
 // the rows, so a tile that holds part of an interval adds its part.
 //
@@ -310,10 +310,13 @@ static_assert(kBC <= 32 * (kWarps3 / 2), "two warps per 32 columns");
 static_assert(kRaw3Bytes % 128 == 0 && (size_t)kZ3 * kB3 * (kB3 + 1) * 4 <= kE3Bytes, "tile layout");
 constexpr size_t kSmem3 = 128 + kRaw3Bytes + kE3Bytes;
 
-// A column half whose largest window of rows exceeds its smallest nonzero one by this factor is
-// summed row by row (window: four rows, one row on panels with fewer than two rows per voxel, so that
-// it is no longer than what a voxel sees).
-constexpr float kWideRatio = 1024.f;  // (clinical pair with noise, 256 / 512 / 1024 / 2048: 17.4 / 17.1 / 16.9 / 16.8 ms)
+// A column half in which a window of rows is smaller (and not zero) by more than 2^kWideLog2 than one
+// nearer to the middle row, where the sums start, is summed row by row. Window: the |p| of four rows
+// (the outermost: up to seven), of one row on panels with fewer than two rows per voxel, so that it is
+// hardly longer than what a voxel sees, and in halves of fewer than eight rows. Clinical adjoint with 2^8 / 2^9 / 2^10 / 2^11,
+// before the groups' loads were batched: projections of a phantom 10.04 / 9.95 / 9.85 / 9.73 ms, with counting
+// noise 10.35 / 10.1 / 9.88 / 9.69, even data 9.3; now with 2^10 9.73, 9.76 and 9.19.
+constexpr int kWideLog2 = 10;
 
 // Columns [u0, u1] and rows [v0, v1] of one angle that reach a brick.
 struct AngleSpan {
@@ -466,32 +469,49 @@ __global__ void __launch_bounds__(kThreads3, 3)
                     const int c = (warp >> 1) * 32 + lane;
                     if (c < nc) {
                         float s0 = 0.f, s1 = 0.f, rr;
-                        // largest window of |p|, and the bits of the smallest nonzero one less 1
-                        float hi = 0.f;
-                        unsigned lo = 0xffffffffu;
-                        auto windows = [&](int rows, auto row) {
-                            auto close = [&](float w) {
-                                hi = fmaxf(hi, w);
-                                lo = __viaddmin_u32(__float_as_uint(w), 0xffffffffu, lo);
-                            };
+                        // the bits of the largest window so far over 2^kWideLog2, and of the smallest one
+                        // that is not zero, less 1
+                        int small = 0;
+                        unsigned least = 0xffffffffu;
+                        auto close = [&](float w) {
+                            const unsigned bits = __float_as_uint(w);
+                            odd |= bits - 1u < (unsigned)small;
+                            small = __viaddmax_s32((int)bits, -(kWideLog2 << 23), small);
+                            least = __viaddmin_u32(bits, 0xffffffffu, least);
+                        };
+                        // groups of four rows: loads first (the sums' stores could alias them), then the sums;
+                        // the rows left over join the last window (fewer would be small by chance)
+                        auto windows = [&](int rows, auto load, auto row) {
+                            float w = 0.f;
                             int r = 0;
-#pragma unroll 2
+                            if (WIN != 1 && rows < 8) {  // one window would be all there is: row by row
+#pragma unroll 1
+                                for (; r < rows; ++r) {
+                                    const float p = load(r);
+                                    row(r, p);
+                                    close(fabsf(p));
+                                }
+                                return;
+                            }
+#pragma unroll 1
                             for (; r + 4 <= rows; r += 4) {
-                                float w = 0.f;
+                                float p[4];
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) p[j] = load(r + j);
 #pragma unroll
                                 for (int j = 0; j < 4; ++j) {
-                                    const float p = fabsf(row(r + j));
-                                    if (WIN == 1) close(p);
-                                    else w = j ? w + p : p;
+                                    row(r + j, p[j]);
+                                    if (WIN == 1) close(fabsf(p[j]));
+                                    else w = j ? w + fabsf(p[j]) : fabsf(p[j]);
                                 }
                                 if (WIN != 1) close(w);
                             }
-                            float w = 0.f;
 #pragma unroll 1
                             for (; r < rows; ++r) {
-                                const float p = fabsf(row(r));
-                                if (WIN == 1) close(p);
-                                else w += p;
+                                const float p = load(r);
+                                row(r, p);
+                                if (WIN == 1) close(fabsf(p));
+                                else w += fabsf(p);
                             }
                             if (WIN != 1) close(w);
                         };
@@ -499,29 +519,28 @@ __global__ void __launch_bounds__(kThreads3, 3)
                             const float *src = raw + c + (h - 1) * kBC;
                             float2 *dst = E + c + (h - 1) * kEP;
                             rr = 1.f;
-                            windows(h, [&](int r) {
-                                const float p = src[-r * kBC];
+                            windows(h, [&](int r) { return src[-r * kBC]; }, [&](int r, float p) {
                                 s0 -= p;
                                 s1 = fmaf(rr, p, s1);
                                 rr += 1.f;
                                 dst[-r * kEP] = make_float2(s0, s1);
-                                return p;
                             });
                         } else {
                             const float *src = raw + c + h * kBC;
                             float2 *dst = E + c + h * kEP;
                             rr = 0.f;
                             dst[0] = make_float2(0.f, 0.f);
-                            windows(nr - h, [&](int r) {
-                                const float p = src[r * kBC];
+                            windows(nr - h, [&](int r) { return src[r * kBC]; }, [&](int r, float p) {
                                 s0 += p;
                                 s1 = fmaf(rr, p, s1);
                                 rr += 1.f;
                                 dst[(r + 1) * kEP] = make_float2(s0, s1);
-                                return p;
                             });
                         }
-                        odd = !all_finite(s0, s1) || hi > kWideRatio * __uint_as_float(lo + 1u);
+                        // where the panel or the tile cuts the brick's rows, a large last window may have
+                        // small rows behind its pixel that no window shows: there its order does not matter
+                        const bool cut = warp & 1 ? v0 > cur.v0 || v0 == 0 : v0 + nr <= cur.v1 || v0 + nr == nv;
+                        odd = odd || !all_finite(s0, s1) || (cut && least < (unsigned)small);
                         wide[warp & 1][c] = odd;
                     }
                 }

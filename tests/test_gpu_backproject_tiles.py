@@ -116,3 +116,22 @@ def test_smooth_projections_to_a_few_roundings(name):
     p = p.float()[None].contiguous()
     got, ref = P.back_project(geom, p), P.back_project(geom, p.double())
     assert float((got.double() - ref).norm()) <= 1e-6 * float(ref.norm())
+
+
+@pytest.mark.parametrize("name", ["fine_panel", "eight_per_part", "nu_113"])
+@pytest.mark.parametrize("rows", [(0, 1), (2, 3), (-2, -1), (-4, -3)])
+def test_large_pixels_near_the_panel_edges(name, rows):
+    """A large pixel in one of the last rows of the panel (or of a tile of a finer panel) has no full window
+    of rows behind it; the voxels that only see those rows keep their value all the same."""
+    geom = P.Geometry(CASES[name])
+    na, nv, nu = geom.proj_shape
+    y = torch.as_tensor(I.random_volume((1,) + geom.proj_shape, 9), device="cuda").abs() + 0.1
+    clean = P.back_project(geom, y)
+    step = 52 if name == "fine_panel" else nv     # (tiles of 52 rows)
+    for row in rows:
+        hot = torch.zeros_like(y)
+        hot[0, :, row % step::step, nu // 5::max(1, nu // 4)] = 1.0
+        got = P.back_project(geom, torch.where(hot > 0, torch.full_like(y, 1e6), y))
+        far = (P.back_project(geom, hot) == 0) & (P.back_project(geom, hot.double()) == 0) & (clean > 0.01 * clean.max())
+        assert int(far.sum()) > 300
+        assert float(((got[far] - clean[far]).abs() / clean[far]).max()) <= 1e-5
