@@ -467,11 +467,11 @@ def report(args, geom, world, S_fwd, samples_step, value, ms, ms_fwd, ms_adj, e2
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch, from one ncu
 # --set full capture of the clinical workload with the current kernels; None elsewhere
 # and whenever the kernel changes after the capture.
-MEASURED_TRAFFIC = {"clinical": {"back_project": 1309.8e6 + 38.6e6, "forward_project": 132.9e6 + 280.1e6}}
+MEASURED_TRAFFIC = {"clinical": {"back_project": 1426.2e6 + 39.0e6, "forward_project": 133.1e6 + 280.5e6}}
 # The binding on-chip level's throughput from the same captures: the projector kernels are
 # bound by SM instruction issue, so this is sm__throughput.avg.pct_of_peak_sustained_elapsed
-# (issue active: forward 80.6 %, adjoint 65.9 %). Same validity rule as the traffic.
-MEASURED_SM_THROUGHPUT_PCT = {"clinical": {"back_project": 62.0, "forward_project": 80.5}}
+# (issue active: forward 79.7 %, adjoint 67.5 %). Same validity rule as the traffic.
+MEASURED_SM_THROUGHPUT_PCT = {"clinical": {"back_project": 64.1, "forward_project": 79.6}}
 
 
 def launches_per_step(geom) -> int:

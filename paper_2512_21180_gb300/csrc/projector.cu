@@ -279,10 +279,10 @@ __global__ void __launch_bounds__(256) k_backproject(GeomDev g, const T *__restr
 // sums start at the tile's middle row h and run outwards, so
 // they span at most half a tile (26 rows) of one column: FP32 rounding stays that of a
 // short sum, and the measured error against 64 bits is the row-by-row kernel's (clinical
-// 3.3e-7 against 3.5e-7). Bounded by instruction issue (66 % of the issue slots; the rest
-// mostly the two barriers of a tile, 24 % of the stalls): about 3/4 of the instructions are the
+// 3.3e-7 against 3.5e-7). Bounded by instruction issue (68 % of the issue slots; the rest
+// mostly the two barriers of a tile, 27 % of the stalls): about 3/4 of the instructions are the
 // intervals, 1/6 the prefix sums. Back projection by CUDA events, row by row -> now:
-// clinical 17.4 -> 9.73 ms, 2 x 128^3 / 200 angles 3.79 -> 1.70 ms, 64^3 / 64 angles 126 -> 54 us.
+// clinical 17.4 -> 9.56 ms, 2 x 128^3 / 200 angles 3.79 -> 1.68 ms, 64^3 / 64 angles 126 -> 54 us.
 //
 // A prefix sum keeps the rounding of every row on its way, so a column half that is not finite or
 // spans too wide a range (kWideLog2) is summed row by row instead, over the same intervals: a large,
@@ -291,8 +291,7 @@ __global__ void __launch_bounds__(256) k_backproject(GeomDev g, const T *__restr
 // their background do not touch, 100 angles: 8.6e-6 of its value against 3.7e-6 without them; with prefix
 // sums everywhere 8e-5 at 10^4 and 6e-3 at 10^6). Such columns lie
 // at the edges of the body, where a tile's middle is inside it: 0.1 % of the column halves of a phantom's
-// projections, which cost the clinical adjoint 6 %.
-// They are read from the landing box, so the next one is sent for after them. A brick
+// projections, which cost the clinical adjoint 6 %. They are read from the landing box, so the next one is sent for after them. A brick
 // whose footprint exceeds the tile takes several tiles per angle: the intervals are linear in
 // the rows, so a tile that holds part of an interval adds its part.
 //
@@ -315,7 +314,7 @@ constexpr size_t kSmem3 = 128 + kRaw3Bytes + kE3Bytes;
 // (the outermost: up to seven), of one row on panels with fewer than two rows per voxel, so that it is
 // hardly longer than what a voxel sees, and in halves of fewer than eight rows. Clinical adjoint with 2^8 / 2^9 / 2^10 / 2^11,
 // before the groups' loads were batched: projections of a phantom 10.04 / 9.95 / 9.85 / 9.73 ms, with counting
-// noise 10.35 / 10.1 / 9.88 / 9.69, even data 9.3; now with 2^10 9.73, 9.76 and 9.19.
+// noise 10.35 / 10.1 / 9.88 / 9.69, even data 9.3; now with 2^10 9.75, 9.79 and 9.22.
 constexpr int kWideLog2 = 10;
 
 // Columns [u0, u1] and rows [v0, v1] of one angle that reach a brick.

@@ -31,9 +31,10 @@
 // finite (a NaN or infinite voxel in a level that only some of the rows use) every ray is
 // summed again from its own samples. Sums run per chunk and then over chunks, which keeps the
 // rounding of a ray well below one long sum's: error against 64 bits 1.5e-7 at the clinical size
-// (7.4e-7 with one running sum). Bounded by instruction issue (78 % of issue slots). Forward
-// projection by CUDA events, two rays per thread -> four: clinical 14.9 -> 7.23 ms, 2 x 128^3 /
-// 200 angles 2.07 -> 1.01 ms, 181 x 167 x 93 / 150 angles 2.10 -> 0.90 ms, 64^3 / 64 angles 48 -> 31 us.
+// (7.4e-7 with one running sum). Bounded by instruction issue (80 % of issue slots). Forward
+// projection by CUDA events, two rays per thread -> four: clinical 14.9 -> 7.42 ms, 2 x 128^3 /
+// 200 angles 2.07 -> 1.06 ms, 181 x 167 x 93 / 150 angles 2.10 -> 0.92 ms, 64^3 / 64 angles 48 -> 31 us (started
+// from L_0: clinical 7.32 ms).
 #include <cudaTypedefs.h>
 
 #include <algorithm>

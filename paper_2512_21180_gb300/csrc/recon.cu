@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(128) k_fdk_ramp(const float *__restrict__ q0, 
 // A row with a non-finite value stays out of the transform and is summed tap by tap; rows of unequal
 // size are brought to one (exactly, by powers of two), so that a row's rounding is relative to its own
 // largest value (unscaled, a partner 10^3 times larger left 2.7e-5 of the row's). Clinical scan
-// (153,600 rows of 912): 1.10 ms, against 7.65 ms for weighting, clearing and the direct filter of
+// (153,600 rows of 912): 1.15 ms, against 7.65 ms for weighting, clearing and the direct filter of
 // k_fdk_ramp with its bank conflicts.
 
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(N / 8, N <= 1024 ? 8 : N == 2048 ? 4 : 2)
 // the L1 sectors). Bounded by instruction issue and load latency, hence the packed pairs, the early
 // end of runs off the panel, and runs that lie inside it without tests (their loads overlap).
 // Clinical scan: 5.57 -> 3.1 ms (tests on every voxel 3.6). 4 CTAs per SM of 64 registers: the whole
-// call 4.28 ms, with 3 / 5 / 6 of them 4.49 / 4.46 / 4.61.
+// call 4.28 ms, with 3 / 5 / 6 of them 4.49 / 4.46 / 4.61 (before the filter's row scaling, 0.05 ms).
 constexpr int kFdkZ = 8;
 __global__ void __launch_bounds__(256, 4) k_fdk_backproject(const float *__restrict__ q, const float2 *__restrict__ cs,
                                                          float *__restrict__ vol, int nx, int ny, int nz, int na, int nue,
